@@ -30,22 +30,13 @@ constexpr int BM = 128;  // rows per tile (UMMA M)
 constexpr int BK = 64;   // K elements per pipeline stage (one 128-byte row)
 constexpr int UK = 16;   // K per tcgen05.mma of kind::f16
 
-enum { EPI_BIAS_GELU = 0, EPI_BIAS = 1, EPI_GELU_GRAD = 2, EPI_F32 = 3 };
-
 struct GemmEpi {
     int M, N;                 // valid rows / columns of C
     int kb_total;             // K blocks of BK
     int kb_per_split;         // K blocks per blockIdx.z
-    const float* bias;        // [N]
-    __nv_bfloat16* out_bf16;  // [M][ld_bf16]
-    int ld_bf16;
-    __nv_bfloat16* out_t;     // [N][ld_t] (transposed copy)
-    int ld_t;
-    float* out_f32;           // [M][ld_f32] (+ blockIdx.z * split_stride for EPI_F32)
+    float* out_f32;           // [M][ld_f32] + blockIdx.z * split_stride
     int ld_f32;
     long long split_stride;
-    const float* zin;         // [M][ld_z]: pre-activation for GELU'
-    int ld_z;
     unsigned* err;
 };
 
@@ -58,43 +49,11 @@ struct GemmEpi {
 // approximations, which add a few 1e-7: far below the BF16 rounding of the
 // activations (2^-9 relative).  The GELU epilogue bounds the fused forward
 // pass; this form takes about half the instructions of the library erff.
-// Also returns exp(-z^2 / 2) for the derivative.
-__device__ __forceinline__ float phi_lower(float z, float* gauss)
-{
-    const float az = fabsf(z);
-    const float t = __fdividef(1.0f, fmaf(0.23164190f, az, 1.0f));  // p / sqrt 2 = 0.3275911 / 1.41421356
-    float poly = fmaf(t, 0.5307027145f, -0.7265760135f);            // a_k / 2
-    poly = fmaf(t, poly, 0.7107068705f);
-    poly = fmaf(t, poly, -0.142248368f);
-    poly = fmaf(t, poly, 0.127414796f);
-    poly *= t;
-    const float e = __expf(-0.5f * z * z);
-    *gauss = e;
-    return poly * e;
-}
-
-// GELU(z) = z Phi(z) and its derivative Phi(z) + z phi(z), phi the standard
-// normal density, with Phi(z) = 1 - Phi(-z) for z >= 0.
-__device__ __forceinline__ float gelu_f(float z)
-{
-    float e;
-    const float lt = phi_lower(z, &e);
-    return z * (z >= 0.0f ? 1.0f - lt : lt);
-}
-
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    float e;
-    const float lt = phi_lower(z, &e);
-    return (z >= 0.0f ? 1.0f - lt : lt) + z * e * 0.39894228040143268f;
-}
-
-// GELU of two values with the packed FP32x2 instructions (the fused
-// forward's epilogue): the same formula as gelu_f, with
-// exp(-z^2 / 2) = 2^(-z^2 log2(e) / 2) on the hardware base-2 exponential
-// and Phi(z) = 1/2 + sign(z) (1/2 - Phi(-|z|)), the sign bit of z moved onto
-// the bracket, so that each step but the reciprocal and the exponential
-// works on both values at once.
+//
+// Two values at a time with the packed FP32x2 instructions: exp(-z^2 / 2) =
+// 2^(-z^2 log2(e) / 2) on the hardware base-2 exponential and Phi(z) = 1/2 +
+// sign(z) (1/2 - Phi(-|z|)), the sign bit of z moved onto the bracket, so
+// that each step but the reciprocal and the exponential works on both.
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -102,133 +61,92 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
-__device__ __forceinline__ float2 gelu2_f(float2 z)
+// Phi(z); gauss = exp(-z^2 / 2).
+__device__ __forceinline__ float2 phi2_f(float2 z, float2& gauss)
 {
     const float2 az = make_float2(fabsf(z.x), fabsf(z.y));
-    const float2 d = __ffma2_rn(make_float2(0.23164190f, 0.23164190f), az, make_float2(1.0f, 1.0f));
+    const float2 d = __ffma2_rn(make_float2(0.23164190f, 0.23164190f), az, make_float2(1.0f, 1.0f));  // p / sqrt 2
     const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
     float2 poly = __ffma2_rn(t, make_float2(0.5307027145f, 0.5307027145f), make_float2(-0.7265760135f, -0.7265760135f));
-    poly = __ffma2_rn(t, poly, make_float2(0.7107068705f, 0.7107068705f));
+    poly = __ffma2_rn(t, poly, make_float2(0.7107068705f, 0.7107068705f));  // a_k / 2
     poly = __ffma2_rn(t, poly, make_float2(-0.142248368f, -0.142248368f));
     poly = __ffma2_rn(t, poly, make_float2(0.127414796f, 0.127414796f));
     poly = __fmul2_rn(poly, t);
     // -z^2 log2(e) / 2
     const float2 a = __fmul2_rn(__fmul2_rn(z, make_float2(-0.72134752f, -0.72134752f)), z);
-    const float2 e = make_float2(ex2_approx(a.x), ex2_approx(a.y));
-    const float2 lt = __fmul2_rn(poly, e);                                              // Phi(-|z|)
+    gauss = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+    const float2 lt = __fmul2_rn(poly, gauss);                                              // Phi(-|z|)
     const float2 hb = __ffma2_rn(lt, make_float2(-1.0f, -1.0f), make_float2(0.5f, 0.5f));  // 1/2 - Phi(-|z|)
     const float2 sh = make_float2(__uint_as_float(__float_as_uint(hb.x) ^ (__float_as_uint(z.x) & 0x80000000u)),
                                   __uint_as_float(__float_as_uint(hb.y) ^ (__float_as_uint(z.y) & 0x80000000u)));
-    return __fmul2_rn(z, __fadd2_rn(sh, make_float2(0.5f, 0.5f)));
+    return __fadd2_rn(sh, make_float2(0.5f, 0.5f));
+}
+
+// GELU(z) = z Phi(z).
+__device__ __forceinline__ float2 gelu2_f(float2 z)
+{
+    float2 gauss;
+    const float2 phi = phi2_f(z, gauss);
+    return __fmul2_rn(z, phi);
+}
+
+// GELU'(z) = Phi(z) + z phi(z), phi the standard normal density.
+__device__ __forceinline__ float2 gelu_grad2_f(float2 z)
+{
+    float2 gauss;
+    const float2 phi = phi2_f(z, gauss);
+    return __ffma2_rn(__fmul2_rn(z, gauss), make_float2(0.39894228040143268f, 0.39894228040143268f), phi);
 }
 
 __global__ void k_debug_gelu(const float* __restrict__ z, int n, int grad, float* __restrict__ out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    if (grad == 2) {
-        out[i] = gelu2_f(make_float2(z[i], 0.0f)).x;
-        return;
-    }
-    out[i] = grad ? gelu_grad_f(z[i]) : gelu_f(z[i]);
+    const float2 zz = make_float2(z[i], 0.0f);
+    out[i] = grad == 1 ? gelu_grad2_f(zz).x : gelu2_f(zz).x;
 }
 
 // Epilogue, in column chunks of EC (32, or NT when NT < 32), through shared
-// memory so that every global store is a coalesced row segment:
-//   1. each thread (one accumulator row) loads EC columns from TMEM and
-//      writes them, plus the bias where the epilogue adds one, to the FP32
-//      staging tile F[128][EC + 4];
-//   2. the CTA walks F with 4 consecutive columns per thread (EC / 4
-//      threads per row): GELU / GELU' (reading the pre-activation as a
-//      coalesced float4), BF16 casts and row stores; the BF16 values of the
-//      transposed copy go to T[EC][128 + 8];
-//   3. the CTA writes T as rows of the transposed output.
+// memory so that every global store is a coalesced row segment: each thread
+// (one accumulator row) writes EC columns from TMEM to the FP32 staging tile
+// F[128][EC + 4], then the CTA walks F with 4 consecutive columns per thread.
 template <int NT>
 struct EpiShape {
     static constexpr int EC = NT < 32 ? NT : 32;   // columns per chunk
     static constexpr int FLD = EC + 4;               // F row stride (floats)
-    static constexpr int TLD = BM + 8;               // T row stride (BF16)
-    static constexpr uint32_t BYTES = BM * FLD * 4 + EC * TLD * 2;
+    static constexpr uint32_t BYTES = BM * FLD * 4;
 };
 
-template <int NT, int EPI>
+template <int NT>
 __device__ __forceinline__ void gemm_epilogue(const GemmEpi& e, uint32_t tmem, int m0, int n0, uint8_t* stage)
 {
     using S = EpiShape<NT>;
-    constexpr int EC = S::EC, FLD = S::FLD, TLD = S::TLD;
+    constexpr int EC = S::EC, FLD = S::FLD;
     float* F = reinterpret_cast<float*>(stage);
-    __nv_bfloat16* T = reinterpret_cast<__nv_bfloat16*>(stage + BM * FLD * 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r_own = warp * 32 + lane;
-    const bool has_t = (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_GRAD) && e.out_t != nullptr;
-    constexpr int TPR = EC / 4;          // threads per row in phase 2
+    constexpr int TPR = EC / 4;          // threads per row
     constexpr int RPP = 128 / TPR;       // rows per pass of the CTA
 #pragma unroll 1
     for (int c0 = 0; c0 < NT; c0 += EC) {
-        // ---- 1: TMEM -> F (row per thread)
 #pragma unroll
         for (int h = 0; h < EC; h += 16) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + h), v);
-            if (EPI == EPI_BIAS_GELU || EPI == EPI_BIAS) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int n = n0 + c0 + h + j;
-                    v[j] += n < e.N ? __ldg(e.bias + n) : 0.0f;
-                }
-            }
             // float4 stores: the 8 lanes of one store phase hit 32 distinct banks
 #pragma unroll
             for (int j = 0; j < 16; j += 4)
                 *reinterpret_cast<float4*>(F + r_own * FLD + h + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         }
         __syncthreads();
-        // ---- 2: coalesced row segments
         const int cq = (threadIdx.x % TPR) * 4;
         const int n = n0 + c0 + cq;
 #pragma unroll 1
         for (int r = threadIdx.x / TPR; r < BM; r += RPP) {
             const int row = m0 + r;
             const float4 x = *reinterpret_cast<const float4*>(F + r * FLD + cq);
-            if (row >= e.M || n >= e.N) continue;
-            if (EPI == EPI_F32) {
+            if (row < e.M && n < e.N)
                 *reinterpret_cast<float4*>(e.out_f32 + (size_t)blockIdx.z * e.split_stride + (size_t)row * e.ld_f32 + n) = x;
-            } else if (EPI == EPI_BIAS) {
-                *reinterpret_cast<float4*>(e.out_f32 + (size_t)row * e.ld_f32 + n) = x;
-            } else {
-                float4 o;
-                if (EPI == EPI_BIAS_GELU) {
-                    if (e.out_f32) *reinterpret_cast<float4*>(e.out_f32 + (size_t)row * e.ld_f32 + n) = x;
-                    o = make_float4(gelu_f(x.x), gelu_f(x.y), gelu_f(x.z), gelu_f(x.w));
-                } else {  // EPI_GELU_GRAD
-                    const float4 z = __ldg(reinterpret_cast<const float4*>(e.zin + (size_t)row * e.ld_z + n));
-                    o = make_float4(x.x * gelu_grad_f(z.x), x.y * gelu_grad_f(z.y), x.z * gelu_grad_f(z.z),
-                                    x.w * gelu_grad_f(z.w));
-                }
-                const __nv_bfloat162 lo = __floats2bfloat162_rn(o.x, o.y), hi = __floats2bfloat162_rn(o.z, o.w);
-                uint2 pk;
-                pk.x = *reinterpret_cast<const unsigned*>(&lo);
-                pk.y = *reinterpret_cast<const unsigned*>(&hi);
-                *reinterpret_cast<uint2*>(e.out_bf16 + (size_t)row * e.ld_bf16 + n) = pk;
-                if (has_t) {
-                    T[(cq + 0) * TLD + r] = lo.x;
-                    T[(cq + 1) * TLD + r] = lo.y;
-                    T[(cq + 2) * TLD + r] = hi.x;
-                    T[(cq + 3) * TLD + r] = hi.y;
-                }
-            }
-        }
-        if (has_t) {
-            __syncthreads();
-            // ---- 3: transposed rows out_t[n][m0 .. m0+127], 8 BF16 per store
-#pragma unroll 1
-            for (int t = threadIdx.x; t < EC * (BM / 8); t += 128) {
-                const int c = t / (BM / 8), r8 = (t % (BM / 8)) * 8;
-                const int nn = n0 + c0 + c, row = m0 + r8;
-                if (nn < e.N && row < e.M)
-                    *reinterpret_cast<uint4*>(e.out_t + (size_t)nn * e.ld_t + row) =
-                        *reinterpret_cast<const uint4*>(T + c * TLD + r8);
-            }
         }
         __syncthreads();
     }
@@ -251,7 +169,7 @@ struct GemmSmem {
 // w owns rows 32w .. 32w+31) for the epilogue.  Every wait is bounded; on a
 // timeout the kernel records SPH_DEV_TIMEOUT, lets its own copies land,
 // frees its tensor memory and returns.
-template <int NT, int EPI, int STAGES>
+template <int NT, int STAGES>
 __global__ void __launch_bounds__(128, 2)
 k_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, GemmEpi e)
 {
@@ -330,7 +248,7 @@ k_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtenso
     tc_fence_after();
     // the CTA agrees on ok, so that the barriers inside are reached by all
     if (__syncthreads_and(ok ? 1 : 0))
-        gemm_epilogue<NT, EPI>(e, tmem, m0, n0, smem_raw + (tiles - raw));
+        gemm_epilogue<NT>(e, tmem, m0, n0, smem_raw + (tiles - raw));
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, L::TMEM_COLS);
@@ -371,30 +289,27 @@ static cudaError_t make_map(CUtensorMap* map, const void* ptr, int rows, int col
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int NT, int EPI>
+template <int NT>
 static cudaError_t launch_gemm_t(const CUtensorMap& ma, const CUtensorMap& mb, const GemmEpi& e, int splits,
                                  cudaStream_t s)
 {
-    // 128-wide tiles with a short K (the layers): 3 stages (96 KB) so that two
-    // CTAs share an SM and one's epilogue overlaps the other's main loop;
-    // the weight-gradient products (long K over the batch) keep a deeper ring
-    constexpr int STAGES = NT >= 256 ? 4 : (NT >= 128 ? (EPI == EPI_F32 ? 6 : 3) : 6);
+    constexpr int STAGES = NT >= 256 ? 4 : 6;
     using L = GemmSmem<NT, STAGES>;
     static bool attr = false;
     if (!attr) {
-        cudaError_t r = cudaFuncSetAttribute(k_gemm<NT, EPI, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t r = cudaFuncSetAttribute(k_gemm<NT, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)L::TOTAL);
         if (r != cudaSuccess) return r;
         attr = true;
     }
     dim3 grid((e.M + BM - 1) / BM, (e.N + NT - 1) / NT, splits);
-    k_gemm<NT, EPI, STAGES><<<grid, 128, L::TOTAL, s>>>(ma, mb, e);
+    k_gemm<NT, STAGES><<<grid, 128, L::TOTAL, s>>>(ma, mb, e);
     return cudaGetLastError();
 }
 
 // C[M][N] = A[M][K] . B[N][K]^T; A, B row-major BF16 with leading
 // dimensions lda, ldb (elements, multiples of 8).  NT chooses the N tile.
-static cudaError_t gemm(int NT, int EPI, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
+static cudaError_t gemm(int NT, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M,
                         int N, int K, int splits, GemmEpi e, cudaStream_t s, long long* launches)
 {
     CUtensorMap ma, mb;
@@ -409,15 +324,9 @@ static cudaError_t gemm(int NT, int EPI, const __nv_bfloat16* A, int lda, const 
     e.kb_per_split = (e.kb_total + splits - 1) / splits;
     splits = (e.kb_total + e.kb_per_split - 1) / e.kb_per_split;
     ++*launches;
-#define SPH_GEMM_CASE(nt, epi) \
-    if (NT == nt && EPI == epi) return launch_gemm_t<nt, epi>(ma, mb, e, splits, s);
-    SPH_GEMM_CASE(128, EPI_BIAS_GELU)
-    SPH_GEMM_CASE(16, EPI_BIAS)
-    SPH_GEMM_CASE(128, EPI_GELU_GRAD)
-    SPH_GEMM_CASE(128, EPI_F32)
-    SPH_GEMM_CASE(16, EPI_F32)
-    SPH_GEMM_CASE(256, EPI_F32)
-#undef SPH_GEMM_CASE
+    if (NT == 16) return launch_gemm_t<16>(ma, mb, e, splits, s);
+    if (NT == 128) return launch_gemm_t<128>(ma, mb, e, splits, s);
+    if (NT == 256) return launch_gemm_t<256>(ma, mb, e, splits, s);
     return cudaErrorInvalidValue;
 }
 
@@ -459,96 +368,6 @@ __global__ void k_cast_weights(const float* __restrict__ P, __nv_bfloat16* __res
                 WT[L.w[l] + c * L.out[l] + r] = v;
             }
         }
-    }
-}
-
-// x [B][MLP_IN] -> x^T [MLP_IN][B]
-__global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ x, int rows, int cols, int ld_in,
-                                 __nv_bfloat16* __restrict__ xt, int ld_out)
-{
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        tile[i][threadIdx.x] = (r < rows && c < cols) ? x[(size_t)r * ld_in + c] : __float2bfloat16_rn(0.f);
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) xt[(size_t)c * ld_out + r] = tile[threadIdx.x][i];
-    }
-}
-
-// Upstream gradient of the loss at the output y [B][16] (FP32):
-// phase 0: force loss mean over rows of 1/2 |y[:,0:3] - t[:,0:3]|^2;
-// phase 1: error-head loss mean of 1/2 (y[:,3] - t[:,3])^2;
-// external: dy given (gradient test).  Writes dY and dY^T in BF16 and adds
-// the loss to *loss.
-__global__ void k_output_grad(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ dy_in,
-                              int B, int phase, __nv_bfloat16* __restrict__ dy, __nv_bfloat16* __restrict__ dyt,
-                              int ld_t, float* __restrict__ loss)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (r < B) {
-        for (int c = 0; c < MLP_OUT; ++c) {
-            float g = 0.f;
-            if (dy_in) {
-                g = dy_in[(size_t)r * MLP_OUT + c];
-            } else if ((phase == 0 && c < 3) || (phase == 1 && c == 3)) {
-                const float d = y[(size_t)r * MLP_OUT + c] - t[(size_t)r * 4 + c];
-                l += 0.5f * d * d;
-                g = d / (float)B;
-            }
-            const __nv_bfloat16 gb = __float2bfloat16_rn(g);
-            dy[(size_t)r * MLP_OUT + c] = gb;
-            dyt[(size_t)c * ld_t + r] = gb;
-        }
-    }
-    // block reduction of the loss
-    __shared__ float red[256];
-    red[threadIdx.x] = l;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && loss) atomicAdd(loss, red[0] / (float)B);
-}
-
-// Sum of the split-K partials of a weight gradient into G (FP32).
-__global__ void k_reduce_splits(const float* __restrict__ part, int splits, long long stride, int n,
-                                float* __restrict__ g)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int k = 0; k < splits; ++k) s += part[(size_t)k * stride + t];
-        g[t] = s;
-    }
-}
-
-// Bias gradient: column sums of d [B][cols] (BF16), one thread per column.
-__global__ void k_col_sums(const __nv_bfloat16* __restrict__ d, int B, int cols, int ld, float* __restrict__ g)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float s = 0.f;
-    for (int r = 0; r < B; ++r) s += __bfloat162float(d[(size_t)r * ld + c]);
-    g[c] = s;
-}
-
-// Adam (Kingma & Ba) on the FP32 master parameters [lo, hi).
-__global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ Mo,
-                       float* __restrict__ Vo, int lo, int hi, float lr, float b1, float b2, float eps, float c1,
-                       float c2)
-{
-    for (int t = lo + blockIdx.x * blockDim.x + threadIdx.x; t < hi; t += gridDim.x * blockDim.x) {
-        const float g = G[t];
-        const float m = b1 * Mo[t] + (1.f - b1) * g;
-        const float v = b2 * Vo[t] + (1.f - b2) * g * g;
-        Mo[t] = m;
-        Vo[t] = v;
-        P[t] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
     }
 }
 
@@ -820,6 +639,448 @@ k_mlp_fused(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CU
     if (warp == LOAD_WARP) tmem_dealloc(tmem, 2 * MLP_H);
 }
 
+// ------------------------------------------------------------------ training
+
+// A training step is three launches: k_train_rows (forward and backward
+// through all layers for a few batch rows per CTA), k_train_dw (every
+// layer's weight and bias gradient, split over the batch) and k_train_update
+// (the splits' sum, Adam, the BF16 copies).
+//
+// k_train_rows: one CTA per NB batch rows.  The products run transposed,
+// out^T[feature][row] = W[feature][k] . act[row][k]^T, with the weights as
+// the 128-row A operand (two halves of 256 features) and the CTA's rows as
+// the N dimension, because a training batch is small: 2,048 rows make 64
+// CTAs of 32 rows where 128-row tiles make 16.  Seven steps: layers 0 .. 3,
+// then the backward products through W4, W3, W2.  The rows' activations stay
+// in one shared-memory buffer (K-major 64-column tiles, 128-byte swizzle),
+// each step's epilogue writing its output over its input once the step's
+// MMAs are done; the three layers' pre-activations stay in tensor memory in
+// FP32 (2 NB columns each) until the backward pass takes their GELU', and
+// the other steps share a fourth region.  An epilogue thread owns a feature
+// and a half of the rows, so what the weight gradients contract over the
+// batch ([feature][batch], BF16) is written straight from its registers.
+// The 26 weight tiles (32 KB) stream through a TMA ring ahead of the steps.
+// Every wait is bounded.
+//
+// What bounds it: the chain of seven dependent steps (MMA, epilogue and
+// barrier each), not bandwidth: 0.68 MB of weights per CTA from L2.  A
+// training step of 2,048 rows took 432 us as 26 launches (four 110 us
+// column sums of one thread per column among them).
+namespace train {
+constexpr int STEPS = 7, STAGES = 5, KB_IN = (MLP_IN + BK - 1) / BK, KB_H = MLP_H / BK;
+constexpr uint32_t W_TILE = MLP_H * BK * 2;  // 32 KB: 256 features x 64 BF16
+constexpr int EPI_WARPS = 16, LOAD_WARP = EPI_WARPS, MMA_WARP = EPI_WARPS + 1;
+constexpr int THREADS = 32 * (EPI_WARPS + 2), EPI_THREADS = 32 * EPI_WARPS;
+// K tiles of a step, bytes of one of its weight tiles
+__host__ __device__ constexpr int kblocks(int s) { return s == 0 ? KB_IN : (s == 4 ? 1 : KB_H); }
+__host__ __device__ constexpr uint32_t tile_bytes(int s) { return s == 3 ? MLP_OUT * BK * 2 : W_TILE; }
+
+template <int NB>
+struct Smem {
+    static constexpr uint32_t ACT_TILE = NB * BK * 2;  // NB rows x 64 BF16
+    static constexpr uint32_t RING = KB_IN * ACT_TILE;
+    static constexpr uint32_t BARS = RING + STAGES * W_TILE;
+    // full[STAGES], empty[STAGES], x_full, acc_full, epi_done, then the TMEM slot
+    static constexpr uint32_t TOTAL = 1024 + BARS + 8 * (2 * STAGES + 3) + 16;
+    static constexpr uint32_t TMEM_COLS = 8 * NB;
+};
+}  // namespace train
+
+struct TrainMaps {
+    CUtensorMap w[4];       // W of layers 0 .. 3
+    CUtensorMap wt[3];      // W^T of layers 3, 2, 1 (steps 4, 5, 6)
+};
+
+struct TrainArgs {
+    const float* P;
+    const float* target;    // [B][4], or NULL: the output gradient is given
+    const float* dy;        // [B][16]
+    int B, phase;
+    int trunk;              // 0: stop after the output gradient
+    int ld_t;               // row length of the transposed arrays
+    __nv_bfloat16 *xt, *ht[3], *dt[3], *dyt;
+    float* loss_part;       // two partial losses per CTA
+    unsigned* err;
+};
+
+template <int NB>
+__global__ void __launch_bounds__(train::THREADS, 1)
+k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ TrainMaps maps, TrainArgs a)
+{
+    using namespace train;
+    using S = Smem<NB>;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* gbase = smem_raw + (base - raw);
+    const uint32_t bars = base + S::BARS;
+    auto full = [&](int s) { return bars + 8u * (uint32_t)s; };
+    auto empty = [&](int s) { return bars + 8u * (uint32_t)(STAGES + s); };
+    const uint32_t x_full = bars + 8u * (2 * STAGES), acc_full = x_full + 8u, epi_done = x_full + 16u;
+    const uint32_t tmem_slot = x_full + 24u;
+    uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(gbase + S::BARS + 8 * (2 * STAGES + 3));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row0 = blockIdx.x * NB;
+    const int nsteps = a.trunk ? STEPS : 4;
+    const ParamLayout L;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        mbar_init(x_full, 1);
+        mbar_init(acc_full, 1);
+        mbar_init(epi_done, EPI_THREADS);
+        mbar_fence_init();
+    }
+    if (warp == LOAD_WARP) tmem_alloc(tmem_slot, S::TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot_ptr;
+    // accumulator of a step: layers 0 .. 2 keep theirs, the others share one
+    auto acc_cols = [&](int s) { return tmem + (uint32_t)((s < 3 ? s : 3) * 2 * NB); };
+
+    if (warp == LOAD_WARP) {
+        if (lane == 0) {
+            mbar_expect_tx(x_full, KB_IN * S::ACT_TILE);
+            for (int kb = 0; kb < KB_IN; ++kb) tma_load_2d(&mapX, x_full, base + kb * S::ACT_TILE, kb * BK, row0);
+            int g = 0;
+            bool ok = true;
+            for (int s = 0; s < nsteps && ok; ++s) {
+                const CUtensorMap* map = s < 4 ? &maps.w[s] : &maps.wt[s - 4];
+                for (int kb = 0; kb < kblocks(s); ++kb, ++g) {
+                    const int st = g % STAGES;
+                    if (g >= STAGES && !mbar_wait(empty(st), (uint32_t)((g / STAGES) - 1) & 1u, a.err)) {
+                        ok = false;
+                        break;
+                    }
+                    mbar_expect_tx(full(st), tile_bytes(s));
+                    tma_load_2d(map, full(st), base + S::RING + st * W_TILE, kb * BK, 0);
+                }
+            }
+            if (!ok) {  // let the copies in flight land before the CTA goes away
+                for (int h = (g > STAGES ? g - STAGES : 0); h < g; ++h)
+                    mbar_wait(full(h % STAGES), (uint32_t)(h / STAGES) & 1u, a.err);
+                mbar_wait(x_full, 0, a.err);
+            }
+        }
+    } else if (warp == MMA_WARP) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16(BM, NB);
+            bool ok = true;
+            int g = 0;
+            for (int s = 0; s < nsteps && ok; ++s) {
+                // step s reads the input tile, or what the epilogue of step s - 1 wrote
+                ok = s == 0 ? mbar_wait(x_full, 0, a.err) : mbar_wait(epi_done, (uint32_t)(s - 1) & 1u, a.err);
+                if (!ok) break;
+                tc_fence_after();
+                for (int kb = 0; kb < kblocks(s); ++kb, ++g) {
+                    const int st = g % STAGES;
+                    if (!mbar_wait(full(st), (uint32_t)(g / STAGES) & 1u, a.err)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t w = base + S::RING + st * W_TILE, act = base + kb * S::ACT_TILE;
+                    // the output layer has 16 features: the other rows of its A
+                    // tile are leftovers of the ring, their lanes never read
+                    const int halves = s == 3 ? 1 : 2, ks = s == 4 ? 1 : BK / UK;
+                    for (int hf = 0; hf < halves; ++hf)
+                        for (int k = 0; k < ks; ++k)
+                            umma_bf16(acc_cols(s) + (uint32_t)(hf * NB), sw128_desc(w + hf * (W_TILE / 2) + k * UK * 2),
+                                      sw128_desc(act + k * UK * 2), idesc, (uint32_t)((kb | k) != 0));
+                    umma_commit(empty(st));
+                }
+                if (!ok) break;
+                umma_commit(acc_full);
+            }
+            if (!ok) umma_commit(acc_full);  // so that the epilogue does not wait for nothing
+        }
+    } else {
+        // warp w reads tensor-memory lanes 32 (w % 4) ..; part w / 4 picks the
+        // feature half and the half of the rows
+        const int q = warp & 3, part = warp >> 2, hf = part >> 1, f = hf * 128 + q * 32 + lane;
+        const int n0 = (part & 1) * (NB / 2);
+        const uint32_t lanes = (uint32_t)(q * 32) << 16;
+        bool ok = mbar_wait(x_full, 0, a.err);
+        if (a.trunk && ok) {  // x^T for the first layer's weight gradient
+            for (int e = threadIdx.x; e < MLP_IN * (NB / 8); e += EPI_THREADS) {
+                const int c = e % MLP_IN, r8 = (e / MLP_IN) * 8;
+                const uint8_t* tile = gbase + (c / BK) * S::ACT_TILE;
+                uint32_t pk[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t lo = *reinterpret_cast<const uint16_t*>(tile + sw128_offset(r8 + 2 * k, c % BK));
+                    const uint32_t hi = *reinterpret_cast<const uint16_t*>(tile + sw128_offset(r8 + 2 * k + 1, c % BK));
+                    pk[k] = lo | (hi << 16);
+                }
+                *reinterpret_cast<uint4*>(a.xt + (size_t)c * a.ld_t + row0 + r8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");  // x read before any epilogue overwrites it
+        for (int s = 0; s < nsteps; ++s) {
+            ok = mbar_wait(acc_full, (uint32_t)s & 1u, a.err);
+            tc_fence_after();
+            if (!ok) break;
+            if (s == 3) {
+                // the output layer: 16 features in the first lanes
+                if (hf == 0 && q == 0) {
+                    float loss = 0.0f;
+                    for (int c = 0; c < NB / 2; c += 16) {
+                        float v[16];
+                        tmem_ld16(acc_cols(3) + lanes + (uint32_t)(n0 + c), v);
+                        if (lane < MLP_OUT) {
+                            const float b = __ldg(a.P + L.b[3] + lane);
+                            uint32_t pk[8];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                const int row = row0 + n0 + c + e;
+                                float g = 0.0f;
+                                if (a.dy) {
+                                    g = __ldg(a.dy + (size_t)row * MLP_OUT + lane);
+                                } else if (a.phase == 0 ? lane < 3 : lane == 3) {
+                                    const float d = v[e] + b - __ldg(a.target + (size_t)row * 4 + lane);
+                                    loss += 0.5f * d * d;
+                                    g = d / (float)a.B;
+                                }
+                                const __nv_bfloat16 gb = __float2bfloat16_rn(g);
+                                const uint16_t u = *reinterpret_cast<const uint16_t*>(&gb);
+                                if (e & 1) pk[e >> 1] |= (uint32_t)u << 16;
+                                else pk[e >> 1] = u;
+                                if (a.trunk)
+                                    *reinterpret_cast<uint16_t*>(gbase + sw128_offset(n0 + c + e, lane)) = u;
+                            }
+                            uint4* o = reinterpret_cast<uint4*>(a.dyt + (size_t)lane * a.ld_t + row0 + n0 + c);
+                            o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                            o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        }
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(FULL, loss, o);
+                    if (lane == 0) a.loss_part[2 * blockIdx.x + part] = loss;
+                }
+            } else {
+                const int l = s < 3 ? s : 6 - s;  // layer whose pre-activation the step meets
+                const float b = __ldg(a.P + L.b[l] + f);
+                __nv_bfloat16* out = s < 3 ? a.ht[l] : a.dt[l];
+                const bool store = a.trunk || s == 2;  // the head alone needs only the last hidden layer
+                for (int c = 0; c < NB / 2; c += 16) {
+                    const uint32_t cols = lanes + (uint32_t)(hf * NB + n0 + c);
+                    float z[16], v[16];
+                    tmem_ld16(acc_cols(l) + cols, z);
+                    if (s > 3) tmem_ld16(acc_cols(s) + cols, v);
+                    uint32_t pk[8];
+#pragma unroll
+                    for (int e = 0; e < 16; e += 2) {
+                        const float2 zz = __fadd2_rn(make_float2(z[e], z[e + 1]), make_float2(b, b));
+                        const float2 r = s < 3 ? gelu2_f(zz) : __fmul2_rn(make_float2(v[e], v[e + 1]), gelu_grad2_f(zz));
+                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(r.x, r.y);
+                        pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+                    }
+                    if (store) {
+                        uint4* o = reinterpret_cast<uint4*>(out + (size_t)f * a.ld_t + row0 + n0 + c);
+                        o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                    }
+                    if (s < 6) {  // the next step's operand: (row n0 + c + e, feature f)
+                        uint8_t* tile = gbase + (f / BK) * S::ACT_TILE;
+#pragma unroll
+                        for (int e = 0; e < 16; ++e)
+                            *reinterpret_cast<uint16_t*>(tile + sw128_offset(n0 + c + e, f % BK)) =
+                                (uint16_t)(pk[e >> 1] >> (16 * (e & 1)));
+                    }
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tc_fence_before();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(epi_done) : "memory");
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == LOAD_WARP) tmem_dealloc(tmem, S::TMEM_COLS);
+}
+
+// Weight and bias gradients of every layer: dW[out][in] = dT[out][B] .
+// inT[in][B]^T over a slice of the batch.  blockIdx.x: a tile of 128 outputs
+// x 144 inputs of a layer (two N tiles cover 256 or 272 inputs: 14 tiles in
+// all), blockIdx.y: the slice.  The first N tile also sums dT over its
+// batch rows, the bias gradient, as a product with a tile of ones (16 more
+// accumulator columns).  Partials go to part[slice] in the packed parameter
+// layout.  One kernel for all layers: a product alone would use 16 SMs.
+namespace dw {
+constexpr int NT = 144, STAGES = 4, TILES = 14;
+constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = NT * BK * 2, STAGE = A_BYTES + B_BYTES;
+constexpr uint32_t ONES = STAGES * STAGE, ONES_BYTES = 16 * BK * 2;
+constexpr uint32_t BARS = ONES + ONES_BYTES;
+constexpr uint32_t TOTAL = 1024 + BARS + 8 * (2 * STAGES + 1) + 16;
+constexpr uint32_t TMEM_COLS = 256;
+static_assert(STAGE % 1024 == 0 && ONES_BYTES % 1024 == 0, "operand tiles start on 1024-byte boundaries");
+}  // namespace dw
+
+struct DwMaps {
+    CUtensorMap d[4];   // dT of layers 0 .. 3, boxes of 128 rows
+    CUtensorMap in[4];  // inT of layers 0 .. 3, boxes of 144 rows
+};
+
+__global__ void __launch_bounds__(128)
+k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, int kb_per_split,
+           float* __restrict__ part, unsigned* __restrict__ err)
+{
+    using namespace dw;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* gbase = smem_raw + (base - raw);
+    const uint32_t bars = base + BARS;
+    auto full = [&](int s) { return bars + 8u * (uint32_t)s; };
+    auto empty = [&](int s) { return bars + 8u * (uint32_t)(STAGES + s); };
+    const uint32_t done = bars + 8u * (2 * STAGES), tmem_slot = done + 8u;
+    uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(gbase + BARS + 8 * (2 * STAGES + 1));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = first_tile + (int)blockIdx.x;
+    const int l = tile < 12 ? tile >> 2 : 3, mt = tile < 12 ? (tile >> 1) & 1 : 0, nt = tile & 1;
+    const int m0 = mt * BM, n0 = nt * NT;
+    const int kb0 = blockIdx.y * kb_per_split, nk = min(kb_per_split, kb_total - kb0);
+    const ParamLayout L;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        mbar_init(done, 1);
+        mbar_fence_init();
+    }
+    for (int e = threadIdx.x; e < (int)ONES_BYTES / 4; e += 128)
+        reinterpret_cast<uint32_t*>(gbase + ONES)[e] = 0x3f803f80u;  // BF16 ones (any swizzle is the same)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (warp == 0) tmem_alloc(tmem_slot, TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot_ptr;
+
+    if (warp == 0 && lane == 0) {
+        int issued = 0;
+        bool ok = true;
+        for (int i = 0; i < nk; ++i) {
+            const int s = i % STAGES;
+            if (i >= STAGES && !mbar_wait(empty(s), (uint32_t)((i / STAGES) - 1) & 1u, err)) {
+                ok = false;
+                break;
+            }
+            mbar_expect_tx(full(s), STAGE);
+            tma_load_2d(&maps.d[l], full(s), base + s * STAGE, (kb0 + i) * BK, m0);
+            tma_load_2d(&maps.in[l], full(s), base + s * STAGE + A_BYTES, (kb0 + i) * BK, n0);
+            ++issued;
+        }
+        if (!ok)
+            for (int i = max(0, issued - STAGES); i < issued; ++i)
+                mbar_wait(full(i % STAGES), (uint32_t)(i / STAGES) & 1u, err);
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = umma_idesc_bf16(BM, NT), idesc1 = umma_idesc_bf16(BM, 16);
+        for (int i = 0; i < nk; ++i) {
+            const int s = i % STAGES;
+            if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, err)) break;
+            tc_fence_after();
+            const uint32_t a = base + s * STAGE, b = a + A_BYTES;
+#pragma unroll
+            for (int k = 0; k < BK / UK; ++k) {
+                umma_bf16(tmem, sw128_desc(a + k * UK * 2), sw128_desc(b + k * UK * 2), idesc, (uint32_t)((i | k) != 0));
+                if (nt == 0)
+                    umma_bf16(tmem + NT, sw128_desc(a + k * UK * 2), sw128_desc(base + ONES + k * UK * 2), idesc1,
+                              (uint32_t)((i | k) != 0));
+            }
+            umma_commit(empty(s));
+        }
+        umma_commit(done);
+    }
+    __syncwarp();
+
+    const bool ok = mbar_wait(done, 0, err);
+    tc_fence_after();
+    if (ok) {
+        const int m = m0 + warp * 32 + lane, nin = L.in[l];
+        const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
+        float* out = part + (size_t)blockIdx.y * SPH_MLP_PARAMS;
+        for (int c = 0; c < NT && n0 + c < nin; c += 16) {  // 16-column chunks end with the layer's inputs
+            float v[16];
+            tmem_ld16(row + (uint32_t)c, v);
+            if (m < L.out[l]) {
+                float4* o = reinterpret_cast<float4*>(out + L.w[l] + m * nin + n0 + c);
+#pragma unroll
+                for (int e = 0; e < 16; e += 4) o[e / 4] = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            }
+        }
+        if (nt == 0) {
+            float v[16];
+            tmem_ld16(row + NT, v);
+            if (m < L.out[l]) out[L.b[l] + m] = v[0];
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
+}
+
+// G = the slices' sum, in order; then (adam) the Adam update (Kingma & Ba)
+// of the FP32 master parameters a phase trains, with their BF16 copies W
+// [out][in] and W^T [in][out].  [lo, SPH_MLP_PARAMS): the parameters with
+// partials.  The first thread adds the partial losses.
+struct AdamArgs {
+    float lr, b1, b2, eps, c1, c2;
+    int phase;
+};
+
+__global__ void __launch_bounds__(256)
+k_train_update(const float* __restrict__ part, int splits, int lo, float* __restrict__ G, float* __restrict__ grads,
+               int adam, AdamArgs o, float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo,
+               __nv_bfloat16* __restrict__ W, __nv_bfloat16* __restrict__ WT, const float* __restrict__ loss_part,
+               int nloss, int B, float* __restrict__ loss)
+{
+    const ParamLayout L;
+    const int t = lo + blockIdx.x * 256 + threadIdx.x;
+    if (loss && blockIdx.x == gridDim.x - 1) {  // the last block: few parameters, and the loss
+        __shared__ float red[8];
+        float s = 0.0f;
+        for (int k = threadIdx.x; k < nloss; k += 256) s += loss_part[k];
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(FULL, s, q);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float tot = 0.0f;
+            for (int w = 0; w < 8; ++w) tot += red[w];
+            *loss = tot / (float)B;
+        }
+    }
+    if (t >= SPH_MLP_PARAMS) return;
+    float g = 0.0f;
+    for (int k = 0; k < splits; ++k) g += part[(size_t)k * SPH_MLP_PARAMS + t];
+    G[t] = g;
+    if (grads) grads[t] = g;
+    if (!adam) return;
+    // phase 0 leaves the error head (row 3 of W4, b4[3]), phase 1 trains it alone
+    const bool head = (t >= L.w[3] + 3 * MLP_H && t < L.w[3] + 4 * MLP_H) || t == L.b[3] + 3;
+    if (head != (o.phase == 1)) return;
+    const float m = o.b1 * Mo[t] + (1.f - o.b1) * g;
+    const float v = o.b2 * Vo[t] + (1.f - o.b2) * g * g;
+    Mo[t] = m;
+    Vo[t] = v;
+    const float p = P[t] - o.lr * (m / o.c1) / (sqrtf(v / o.c2) + o.eps);
+    P[t] = p;
+    const int l = t >= L.w[3] ? 3 : (t >= L.w[2] ? 2 : (t >= L.w[1] ? 1 : 0));
+    const int e = t - L.w[l];
+    if (e < L.wn[l]) {
+        const __nv_bfloat16 w = __float2bfloat16_rn(p);
+        W[t] = w;
+        WT[L.w[l] + (e % L.in[l]) * L.out[l] + e / L.in[l]] = w;
+    }
+}
+
 }  // namespace sphk
 
 // ------------------------------------------------------------------ API
@@ -830,21 +1091,26 @@ struct sph_mlp {
     int max_batch;
     float *P, *G, *Mo, *Vo;            // packed parameters, gradients, Adam moments
     __nv_bfloat16 *W, *WT;             // BF16 weights and transposes (packed like P)
-    __nv_bfloat16 *XT;                 // [IN][Bmax]
-    __nv_bfloat16 *H[3], *HT[3];       // [B][H], [H][B]
-    float* Z[3];                       // [B][H]
-    float* Y;                          // [B][16]
-    __nv_bfloat16 *DY, *DYT;           // [B][16], [16][B]
-    __nv_bfloat16 *D[2], *DT[2];       // [B][H], [H][B] (alternating)
-    float* part;                       // split-K partials
+    __nv_bfloat16 *XT, *HT[3];         // transposed input and hidden activations [features][Bmax]
+    __nv_bfloat16 *DT[3], *DYT;        // transposed gradients of the pre-activations and of the output
+    float* part;                       // split-K partials: `splits` packed parameter vectors
+    int splits;
+    float* loss_part;                  // two partial losses per 32 rows
     float* loss;
     unsigned* err;
     long long step;
     long long launches;
+    // tensor maps of the handle's own arrays (built by the first training call)
+    bool maps_ready;
+    TrainMaps tmaps;
+    DwMaps dmaps;
     char msg[512];
 };
 
-static const int SPLITS = 8;
+// Slices of the batch in the weight gradients: up to eight (14 tiles x 8 =
+// 112 CTAs), fewer for small handles so that the partials do not outgrow
+// the activations.
+static int max_splits(int max_batch) { return max_batch >= 1152 ? 8 : 2 + max_batch / 192; }
 
 static int mfail(sph_mlp* m, int code, const char* fmt, ...)
 {
@@ -890,60 +1156,16 @@ static size_t mlp_carve(sph_mlp* m, uintptr_t base)
     m->WT = c.take<__nv_bfloat16>(P);
     m->XT = c.take<__nv_bfloat16>((size_t)MLP_IN * B);
     for (int l = 0; l < 3; ++l) {
-        m->H[l] = c.take<__nv_bfloat16>((size_t)MLP_H * B);
         m->HT[l] = c.take<__nv_bfloat16>((size_t)MLP_H * B);
-        m->Z[l] = c.take<float>((size_t)MLP_H * B);
-    }
-    m->Y = c.take<float>((size_t)MLP_OUT * B);
-    m->DY = c.take<__nv_bfloat16>((size_t)MLP_OUT * B);
-    m->DYT = c.take<__nv_bfloat16>((size_t)MLP_OUT * B);
-    for (int l = 0; l < 2; ++l) {
-        m->D[l] = c.take<__nv_bfloat16>((size_t)MLP_H * B);
         m->DT[l] = c.take<__nv_bfloat16>((size_t)MLP_H * B);
     }
-    m->part = c.take<float>((size_t)SPLITS * MLP_H * MLP_IN);
+    m->DYT = c.take<__nv_bfloat16>((size_t)MLP_OUT * B);
+    m->splits = max_splits(m->max_batch);
+    m->part = c.take<float>((size_t)m->splits * P);
+    m->loss_part = c.take<float>(2 * (B / 32));
     m->loss = c.take<float>(4);
     m->err = c.take<unsigned>(4);
     return (c.off + 255) & ~(uintptr_t)255;
-}
-
-static GemmEpi epi0(sph_mlp* m)
-{
-    GemmEpi e;
-    memset(&e, 0, sizeof(e));
-    e.err = m->err;
-    return e;
-}
-
-// Forward pass of B rows of x (BF16 [B][IN]); keep = 1 also stores the
-// pre-activations and the transposed activations for the backward pass.
-static int mlp_forward(sph_mlp* m, const __nv_bfloat16* x, int B, float* y, bool keep, cudaStream_t s)
-{
-    const ParamLayout L;
-    const __nv_bfloat16* in = x;
-    int ld_in = MLP_IN, k_in = MLP_IN;
-    for (int l = 0; l < 3; ++l) {
-        GemmEpi e = epi0(m);
-        e.bias = m->P + L.b[l];
-        e.out_bf16 = m->H[l];
-        e.ld_bf16 = MLP_H;
-        if (keep) {
-            e.out_f32 = m->Z[l];
-            e.ld_f32 = MLP_H;
-            e.out_t = m->HT[l];
-            e.ld_t = m->max_batch;
-        }
-        MLP_TRY(m, gemm(128, EPI_BIAS_GELU, in, ld_in, m->W + L.w[l], L.in[l], B, MLP_H, k_in, 1, e, s, &m->launches));
-        in = m->H[l];
-        ld_in = MLP_H;
-        k_in = MLP_H;
-    }
-    GemmEpi e = epi0(m);
-    e.bias = m->P + L.b[3];
-    e.out_f32 = y;
-    e.ld_f32 = MLP_OUT;
-    MLP_TRY(m, gemm(16, EPI_BIAS, in, MLP_H, m->W + L.w[3], MLP_H, B, MLP_OUT, MLP_H, 1, e, s, &m->launches));
-    return SPH_OK;
 }
 
 // Inference: the four layers in one launch (k_mlp_fused), 128-row tiles.
@@ -973,54 +1195,96 @@ static int mlp_forward_fused(sph_mlp* m, const __nv_bfloat16* x, int B, float* y
     return SPH_OK;
 }
 
-// Weight and bias gradients of layer l from its output gradient d [B][out]
-// (d^T [out][B] given) and its input^T [in][B].
-static int layer_grads(sph_mlp* m, int l, const __nv_bfloat16* d, const __nv_bfloat16* dt, int ld_d,
-                       const __nv_bfloat16* in_t, int B, cudaStream_t s)
+static int sms_of_device(sph_mlp* m, int* sms)
 {
+    int dev = 0;
+    MLP_TRY(m, cudaGetDevice(&dev));
+    MLP_TRY(m, cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+    return SPH_OK;
+}
+
+static int train_maps(sph_mlp* m)
+{
+    if (m->maps_ready) return SPH_OK;
     const ParamLayout L;
-    const int nout = L.out[l], nin = L.in[l];
-    GemmEpi e = epi0(m);
-    e.out_f32 = m->part;
-    e.ld_f32 = nin;
-    e.split_stride = (long long)nout * nin;
-    const int NT = nin > 256 ? 128 : 256;
-    MLP_TRY(m, gemm(NT, EPI_F32, dt, m->max_batch, in_t, m->max_batch, nout, nin, B, SPLITS, e, s, &m->launches));
-    const int kb = (B + BK - 1) / BK, per = (kb + SPLITS - 1) / SPLITS, splits = (kb + per - 1) / per;
-    k_reduce_splits<<<120, 256, 0, s>>>(m->part, splits, e.split_stride, nout * nin, m->G + L.w[l]);
-    k_col_sums<<<(nout + 127) / 128, 128, 0, s>>>(d, B, nout, ld_d, m->G + L.b[l]);
-    m->launches += 2;
+    for (int l = 0; l < 4; ++l)
+        MLP_TRY(m, make_map(&m->tmaps.w[l], m->W + L.w[l], L.out[l], L.in[l], L.in[l], L.out[l]));
+    for (int l = 3; l > 0; --l)
+        MLP_TRY(m, make_map(&m->tmaps.wt[3 - l], m->WT + L.w[l], L.in[l], L.out[l], L.out[l], L.in[l]));
+    for (int l = 0; l < 4; ++l) {
+        MLP_TRY(m, make_map(&m->dmaps.d[l], l < 3 ? m->DT[l] : m->DYT, L.out[l], m->max_batch, m->max_batch, BM));
+        MLP_TRY(m, make_map(&m->dmaps.in[l], l ? m->HT[l - 1] : m->XT, L.in[l], m->max_batch, m->max_batch, dw::NT));
+    }
+    m->maps_ready = true;
+    return SPH_OK;
+}
+
+template <int NB>
+static int launch_rows(sph_mlp* m, const CUtensorMap& mx, const TrainArgs& a, cudaStream_t s)
+{
+    static bool attr = false;
+    if (!attr) {
+        MLP_TRY(m, cudaFuncSetAttribute(k_train_rows<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)train::Smem<NB>::TOTAL));
+        attr = true;
+    }
+    k_train_rows<NB><<<a.B / NB, train::THREADS, train::Smem<NB>::TOTAL, s>>>(mx, m->tmaps, a);
+    ++m->launches;
     MLP_TRY(m, cudaGetLastError());
     return SPH_OK;
 }
 
-// Backward pass from the output gradient (phase 0 / external: every layer;
-// phase 1: the output layer only).
-static int mlp_backward(sph_mlp* m, int B, bool trunk, cudaStream_t s)
+// Gradients of one batch (targets t: the phase's loss; else the output
+// gradient dy), and with adam the update.
+static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const float* dy, int B, int phase,
+                      float* grads, const AdamArgs* adam, float* loss, cudaStream_t s)
 {
     const ParamLayout L;
-    int rc = layer_grads(m, 3, m->DY, m->DYT, MLP_OUT, m->HT[2], B, s);
-    if (rc != SPH_OK || !trunk) return rc;
-    // d3 = (dY . W4) * gelu'(z3)
-    const __nv_bfloat16* dprev = m->DY;
-    int ld_prev = MLP_OUT, k_prev = MLP_OUT;
-    for (int l = 2; l >= 0; --l) {
-        const int cur = l & 1;
-        GemmEpi e = epi0(m);
-        e.zin = m->Z[l];
-        e.ld_z = MLP_H;
-        e.out_bf16 = m->D[cur];
-        e.ld_bf16 = MLP_H;
-        e.out_t = m->DT[cur];
-        e.ld_t = m->max_batch;
-        MLP_TRY(m, gemm(128, EPI_GELU_GRAD, dprev, ld_prev, m->WT + L.w[l + 1], L.out[l + 1], B, MLP_H, k_prev, 1, e,
-                        s, &m->launches));
-        rc = layer_grads(m, l, m->D[cur], m->DT[cur], MLP_H, l == 0 ? m->XT : m->HT[l - 1], B, s);
-        if (rc != SPH_OK) return rc;
-        dprev = m->D[cur];
-        ld_prev = MLP_H;
-        k_prev = MLP_H;
+    int rc = train_maps(m), sms = 0;
+    if (rc == SPH_OK) rc = sms_of_device(m, &sms);
+    if (rc != SPH_OK) return rc;
+    TrainArgs a;
+    memset(&a, 0, sizeof(a));
+    a.P = m->P;
+    a.target = t;
+    a.dy = dy;
+    a.B = B;
+    a.phase = phase;
+    a.trunk = phase == 0;
+    a.ld_t = m->max_batch;
+    a.xt = m->XT;
+    for (int l = 0; l < 3; ++l) {
+        a.ht[l] = m->HT[l];
+        a.dt[l] = m->DT[l];
     }
+    a.dyt = m->DYT;
+    a.loss_part = m->loss_part;
+    a.err = m->err;
+    // 32 rows a CTA while one wave of CTAs takes the batch (its weights are
+    // streamed once per CTA), 64 beyond
+    const int NB = B <= 32 * sms ? 32 : 64;
+    CUtensorMap mx;
+    MLP_TRY(m, make_map(&mx, x, B, MLP_IN, MLP_IN, NB));
+    rc = NB == 32 ? launch_rows<32>(m, mx, a, s) : launch_rows<64>(m, mx, a, s);
+    if (rc != SPH_OK) return rc;
+    static bool attr = false;
+    if (!attr) {
+        MLP_TRY(m, cudaFuncSetAttribute(k_train_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw::TOTAL));
+        attr = true;
+    }
+    const int kb = B / BK;
+    int splits = m->splits < kb ? m->splits : kb;
+    const int per = (kb + splits - 1) / splits;
+    splits = (kb + per - 1) / per;
+    const int first = phase == 0 ? 0 : 12, lo = phase == 0 ? 0 : L.w[3];
+    k_train_dw<<<dim3(dw::TILES - first, splits), 128, dw::TOTAL, s>>>(m->dmaps, first, kb, per, m->part, m->err);
+    AdamArgs none;
+    memset(&none, 0, sizeof(none));
+    k_train_update<<<(SPH_MLP_PARAMS - lo + 255) / 256, 256, 0, s>>>(
+        m->part, splits, lo, m->G, grads, adam != nullptr, adam ? *adam : none, m->P, m->Mo, m->Vo, m->W, m->WT,
+        m->loss_part, 2 * (B / NB), B, loss);
+    m->launches += 2;
+    MLP_TRY(m, cudaGetLastError());
     return SPH_OK;
 }
 
@@ -1128,19 +1392,7 @@ int sph_mlp_gradients(sph_mlp* m, const void* x, const float* dy, int B, float* 
     int rc = check_batch(m, B);
     if (rc != SPH_OK) return rc;
     if (!x || !dy || !grads || ((uintptr_t)x & 15)) return mfail(m, SPH_ERR_ARG, "bad pointers");
-    cudaStream_t s = (cudaStream_t)stream;
-    dim3 tb(32, 8), tg((MLP_IN + 31) / 32, (B + 31) / 32);
-    k_transpose_bf16<<<tg, tb, 0, s>>>((const __nv_bfloat16*)x, B, MLP_IN, MLP_IN, m->XT, m->max_batch);
-    ++m->launches;
-    rc = mlp_forward(m, (const __nv_bfloat16*)x, B, m->Y, true, s);
-    if (rc != SPH_OK) return rc;
-    k_output_grad<<<(B + 255) / 256, 256, 0, s>>>(m->Y, nullptr, dy, B, 0, m->DY, m->DYT, m->max_batch, nullptr);
-    ++m->launches;
-    MLP_TRY(m, cudaGetLastError());
-    rc = mlp_backward(m, B, true, s);
-    if (rc != SPH_OK) return rc;
-    MLP_TRY(m, cudaMemcpyAsync(grads, m->G, sizeof(float) * SPH_MLP_PARAMS, cudaMemcpyDeviceToDevice, s));
-    return SPH_OK;
+    return train_pass(m, (const __nv_bfloat16*)x, nullptr, dy, B, 0, grads, nullptr, nullptr, (cudaStream_t)stream);
 }
 
 int sph_mlp_train_step(sph_mlp* m, const void* x, const float* target, int B, int phase, float lr,
@@ -1150,45 +1402,15 @@ int sph_mlp_train_step(sph_mlp* m, const void* x, const float* target, int B, in
     if (rc != SPH_OK) return rc;
     if (!x || !target || ((uintptr_t)x & 15)) return mfail(m, SPH_ERR_ARG, "bad pointers");
     if (phase != 0 && phase != 1) return mfail(m, SPH_ERR_ARG, "phase must be 0 or 1");
-    cudaStream_t s = (cudaStream_t)stream;
-    const ParamLayout L;
-    dim3 tb(32, 8), tg((MLP_IN + 31) / 32, (B + 31) / 32);
-    if (phase == 0) {
-        k_transpose_bf16<<<tg, tb, 0, s>>>((const __nv_bfloat16*)x, B, MLP_IN, MLP_IN, m->XT, m->max_batch);
-        ++m->launches;
-    }
-    rc = mlp_forward(m, (const __nv_bfloat16*)x, B, m->Y, true, s);
-    if (rc != SPH_OK) return rc;
-    MLP_TRY(m, cudaMemsetAsync(m->loss, 0, sizeof(float), s));
-    k_output_grad<<<(B + 255) / 256, 256, 0, s>>>(m->Y, target, nullptr, B, phase, m->DY, m->DYT, m->max_batch,
-                                                  m->loss);
-    ++m->launches;
-    MLP_TRY(m, cudaGetLastError());
-    rc = mlp_backward(m, B, phase == 0, s);
-    if (rc != SPH_OK) return rc;
-    ++m->step;
     const float b1 = 0.9f, b2 = 0.999f;
     // bias corrections 1 - beta^t in double (in float32 the difference
     // cancels: 1 - 0.999^t loses most of its digits for small t)
-    const float c1 = (float)(1.0 - pow((double)b1, (double)m->step));
-    const float c2 = (float)(1.0 - pow((double)b2, (double)m->step));
-    if (phase == 0) {
-        // every parameter except the error-head row 3 of W4 and b4[3]
-        k_adam<<<256, 256, 0, s>>>(m->P, m->G, m->Mo, m->Vo, 0, L.w[3] + 3 * MLP_H, lr, b1, b2, 1e-8f, c1, c2);
-        k_adam<<<4, 256, 0, s>>>(m->P, m->G, m->Mo, m->Vo, L.w[3] + 4 * MLP_H, L.b[3] + 3, lr, b1, b2, 1e-8f, c1, c2);
-        k_adam<<<1, 32, 0, s>>>(m->P, m->G, m->Mo, m->Vo, L.b[3] + 4, L.b[3] + MLP_OUT, lr, b1, b2, 1e-8f, c1, c2);
-        m->launches += 3;
-    } else {
-        k_adam<<<1, 256, 0, s>>>(m->P, m->G, m->Mo, m->Vo, L.w[3] + 3 * MLP_H, L.w[3] + 4 * MLP_H, lr, b1, b2, 1e-8f,
-                                 c1, c2);
-        k_adam<<<1, 32, 0, s>>>(m->P, m->G, m->Mo, m->Vo, L.b[3] + 3, L.b[3] + 4, lr, b1, b2, 1e-8f, c1, c2);
-        m->launches += 2;
-    }
-    k_cast_weights<<<256, 256, 0, s>>>(m->P, m->W, m->WT);
-    ++m->launches;
-    MLP_TRY(m, cudaGetLastError());
-    if (loss_out) MLP_TRY(m, cudaMemcpyAsync(loss_out, m->loss, sizeof(float), cudaMemcpyDeviceToDevice, s));
-    return SPH_OK;
+    const double k = (double)(m->step + 1);
+    const AdamArgs adam{lr, b1, b2, 1e-8f, (float)(1.0 - pow((double)b1, k)), (float)(1.0 - pow((double)b2, k)), phase};
+    rc = train_pass(m, (const __nv_bfloat16*)x, target, nullptr, B, phase, nullptr, &adam,
+                    loss_out ? loss_out : m->loss, (cudaStream_t)stream);
+    if (rc == SPH_OK) ++m->step;
+    return rc;
 }
 
 int sph_mlp_status(sph_mlp* m, unsigned* bits, void* stream)
@@ -1227,7 +1449,7 @@ int sph_debug_gemm(const void* A, int lda, const void* B, int ldb, int M, int N,
     e.split_stride = (long long)M * N;
     long long launches = 0;
     const int NT = N <= 16 ? 16 : (N <= 128 ? 128 : 256);
-    cudaError_t r = gemm(NT, EPI_F32, (const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, N, K, splits,
+    cudaError_t r = gemm(NT, (const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, N, K, splits,
                          e, (cudaStream_t)stream, &launches);
     if (r != cudaSuccess) return mfail(nullptr, SPH_ERR_CUDA, "GEMM: %s", cudaGetErrorString(r));
     return SPH_OK;

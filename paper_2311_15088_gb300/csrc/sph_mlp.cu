@@ -786,11 +786,23 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
                     const uint32_t w = base + S::RING + st * W_TILE, act = base + kb * S::ACT_TILE;
                     // the output layer has 16 features: the other rows of its A
                     // tile are leftovers of the ring, their lanes never read
-                    const int halves = s == 3 ? 1 : 2, ks = s == 4 ? 1 : BK / UK;
-                    for (int hf = 0; hf < halves; ++hf)
-                        for (int k = 0; k < ks; ++k)
-                            umma_bf16(acc_cols(s) + (uint32_t)(hf * NB), sw128_desc(w + hf * (W_TILE / 2) + k * UK * 2),
-                                      sw128_desc(act + k * UK * 2), idesc, (uint32_t)((kb | k) != 0));
+                    const uint64_t wd = sw128_desc(w), ad = sw128_desc(act);
+                    // a K step of 16 is 32 bytes, 2 in the descriptor's address
+                    // field; the second half of the features 16 KB, 1024 there
+                    auto issue = [&](int hf, int k) {
+                        umma_bf16(acc_cols(s) + (uint32_t)(hf * NB), wd + (uint64_t)(hf * (int)(W_TILE / 32) + 2 * k),
+                                  ad + (uint64_t)(2 * k), idesc, (uint32_t)((kb | k) != 0));
+                    };
+                    if (s == 4) {  // 16 columns
+                        issue(0, 0);
+                        issue(1, 0);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < BK / UK; ++k) {
+                            issue(0, k);
+                            if (s != 3) issue(1, k);
+                        }
+                    }
                     umma_commit(empty(st));
                 }
                 if (!ok) break;
@@ -801,6 +813,11 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
     } else {
         // warp w reads tensor-memory lanes 32 (w % 4) ..; part w / 4 picks the
         // feature half and the half of the rows
+        constexpr int CH = NB >= 32 ? 16 : 8;  // rows (accumulator columns) per chunk
+        auto tmem_ld = [](uint32_t addr, float (&v)[CH]) {
+            if constexpr (CH == 16) tmem_ld16(addr, v);
+            else tmem_ld8(addr, v);
+        };
         const int q = warp & 3, part = warp >> 2, hf = part >> 1, f = hf * 128 + q * 32 + lane;
         const int n0 = (part & 1) * (NB / 2);
         const uint32_t lanes = (uint32_t)(q * 32) << 16;
@@ -820,22 +837,28 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
             }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");  // x read before any epilogue overwrites it
-        for (int s = 0; s < nsteps; ++s) {
+        // this thread's biases, before the steps' critical path
+        const float bias[3] = {__ldg(a.P + L.b[0] + f), __ldg(a.P + L.b[1] + f), __ldg(a.P + L.b[2] + f)};
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+            if (s >= nsteps) break;
             ok = mbar_wait(acc_full, (uint32_t)s & 1u, a.err);
             tc_fence_after();
             if (!ok) break;
+            uint32_t pk[NB / 2 / CH][CH / 2];
             if (s == 3) {
                 // the output layer: 16 features in the first lanes
                 if (hf == 0 && q == 0) {
                     float loss = 0.0f;
-                    for (int c = 0; c < NB / 2; c += 16) {
-                        float v[16];
-                        tmem_ld16(acc_cols(3) + lanes + (uint32_t)(n0 + c), v);
+#pragma unroll
+                    for (int c = 0; c < NB / 2; c += CH) {
+                        float v[CH];
+                        tmem_ld(acc_cols(3) + lanes + (uint32_t)(n0 + c), v);
                         if (lane < MLP_OUT) {
                             const float b = __ldg(a.P + L.b[3] + lane);
-                            uint32_t pk[8];
+                            uint32_t(&p)[CH / 2] = pk[c / CH];
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) {
+                            for (int e = 0; e < CH; ++e) {
                                 const int row = row0 + n0 + c + e;
                                 float g = 0.0f;
                                 if (a.dy) {
@@ -847,14 +870,11 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
                                 }
                                 const __nv_bfloat16 gb = __float2bfloat16_rn(g);
                                 const uint16_t u = *reinterpret_cast<const uint16_t*>(&gb);
-                                if (e & 1) pk[e >> 1] |= (uint32_t)u << 16;
-                                else pk[e >> 1] = u;
+                                if (e & 1) p[e >> 1] |= (uint32_t)u << 16;
+                                else p[e >> 1] = u;
                                 if (a.trunk)
                                     *reinterpret_cast<uint16_t*>(gbase + sw128_offset(n0 + c + e, lane)) = u;
                             }
-                            uint4* o = reinterpret_cast<uint4*>(a.dyt + (size_t)lane * a.ld_t + row0 + n0 + c);
-                            o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                            o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
                         }
                     }
 #pragma unroll
@@ -863,39 +883,46 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
                 }
             } else {
                 const int l = s < 3 ? s : 6 - s;  // layer whose pre-activation the step meets
-                const float b = __ldg(a.P + L.b[l] + f);
-                __nv_bfloat16* out = s < 3 ? a.ht[l] : a.dt[l];
-                const bool store = a.trunk || s == 2;  // the head alone needs only the last hidden layer
-                for (int c = 0; c < NB / 2; c += 16) {
-                    const uint32_t cols = lanes + (uint32_t)(hf * NB + n0 + c);
-                    float z[16], v[16];
-                    tmem_ld16(acc_cols(l) + cols, z);
-                    if (s > 3) tmem_ld16(acc_cols(s) + cols, v);
-                    uint32_t pk[8];
+                const float b = bias[l];
 #pragma unroll
-                    for (int e = 0; e < 16; e += 2) {
+                for (int c = 0; c < NB / 2; c += CH) {
+                    const uint32_t cols = lanes + (uint32_t)(hf * NB + n0 + c);
+                    float z[CH], v[CH];
+                    tmem_ld(acc_cols(l) + cols, z);
+                    if (s > 3) tmem_ld(acc_cols(s) + cols, v);
+                    uint32_t(&p)[CH / 2] = pk[c / CH];
+#pragma unroll
+                    for (int e = 0; e < CH; e += 2) {
                         const float2 zz = __fadd2_rn(make_float2(z[e], z[e + 1]), make_float2(b, b));
                         const float2 r = s < 3 ? gelu2_f(zz) : __fmul2_rn(make_float2(v[e], v[e + 1]), gelu_grad2_f(zz));
                         const __nv_bfloat162 h2 = __floats2bfloat162_rn(r.x, r.y);
-                        pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-                    }
-                    if (store) {
-                        uint4* o = reinterpret_cast<uint4*>(out + (size_t)f * a.ld_t + row0 + n0 + c);
-                        o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        p[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
                     }
                     if (s < 6) {  // the next step's operand: (row n0 + c + e, feature f)
                         uint8_t* tile = gbase + (f / BK) * S::ACT_TILE;
 #pragma unroll
-                        for (int e = 0; e < 16; ++e)
+                        for (int e = 0; e < CH; ++e)
                             *reinterpret_cast<uint16_t*>(tile + sw128_offset(n0 + c + e, f % BK)) =
-                                (uint16_t)(pk[e >> 1] >> (16 * (e & 1)));
+                                (uint16_t)(p[e >> 1] >> (16 * (e & 1)));
                     }
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_fence_before();
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(epi_done) : "memory");
+            // the transposed copy, off the next step's path (a warp's stores go
+            // to 32 rows and would hold up the operand's)
+            __nv_bfloat16* out = s == 3 ? a.dyt : (s < 3 ? a.ht[s < 3 ? s : 0] : a.dt[s < 4 ? 0 : 6 - s]);
+            const bool mine = s == 3 ? hf == 0 && q == 0 && lane < MLP_OUT : a.trunk || s == 2;
+            if (mine)
+#pragma unroll
+                for (int c = 0; c < NB / 2; c += CH) {
+                    uint4* o = reinterpret_cast<uint4*>(out + (size_t)f * a.ld_t + row0 + n0 + c);
+                    const uint32_t(&p)[CH / 2] = pk[c / CH];
+#pragma unroll
+                    for (int k = 0; k < CH / 8; ++k)
+                        o[k] = make_uint4(p[4 * k], p[4 * k + 1], p[4 * k + 2], p[4 * k + 3]);
+                }
         }
     }
     tc_fence_before();
@@ -1006,20 +1033,33 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
         const int m = m0 + warp * 32 + lane, nin = L.in[l];
         const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
         float* out = part + (size_t)blockIdx.y * SPH_MLP_PARAMS;
-        for (int c = 0; c < NT && n0 + c < nin; c += 16) {  // 16-column chunks end with the layer's inputs
+        // a thread's row goes through shared memory (the idle ring; the odd
+        // number of 16-byte chunks per row spreads a warp's over the banks)
+        // and out as one bulk copy: stored by the warp, 32 rows an instruction
+        constexpr int LD = NT + 4;
+        static_assert(128 * LD * 4 <= STAGES * STAGE, "the rows fit the ring");
+        float* stage = reinterpret_cast<float*>(gbase) + threadIdx.x * LD;
+        const int w = min(NT, nin - n0);  // 16-column chunks end with the layer's inputs
+        for (int c = 0; c < w; c += 16) {
             float v[16];
             tmem_ld16(row + (uint32_t)c, v);
-            if (m < L.out[l]) {
-                float4* o = reinterpret_cast<float4*>(out + L.w[l] + m * nin + n0 + c);
 #pragma unroll
-                for (int e = 0; e < 16; e += 4) o[e / 4] = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-            }
+            for (int e = 0; e < 16; e += 4)
+                *reinterpret_cast<float4*>(stage + c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (m < L.out[l]) {
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out + L.w[l] + m * nin + n0),
+                         "r"(smem_u32(stage)), "r"(w * 4)
+                         : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
         if (nt == 0) {
             float v[16];
             tmem_ld16(row + NT, v);
             if (m < L.out[l]) out[L.b[l] + m] = v[0];
         }
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
@@ -1035,49 +1075,71 @@ struct AdamArgs {
     int phase;
 };
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(128)
 k_train_update(const float* __restrict__ part, int splits, int lo, float* __restrict__ G, float* __restrict__ grads,
                int adam, AdamArgs o, float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo,
                __nv_bfloat16* __restrict__ W, __nv_bfloat16* __restrict__ WT, const float* __restrict__ loss_part,
                int nloss, int B, float* __restrict__ loss)
 {
     const ParamLayout L;
-    const int t = lo + blockIdx.x * 256 + threadIdx.x;
+    const int t = lo + 4 * (int)(blockIdx.x * 128 + threadIdx.x);
     if (loss && blockIdx.x == gridDim.x - 1) {  // the last block: few parameters, and the loss
-        __shared__ float red[8];
+        __shared__ float red[4];
         float s = 0.0f;
-        for (int k = threadIdx.x; k < nloss; k += 256) s += loss_part[k];
+        for (int k = threadIdx.x; k < nloss; k += 128) s += loss_part[k];
 #pragma unroll
         for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(FULL, s, q);
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
         __syncthreads();
         if (threadIdx.x == 0) {
             float tot = 0.0f;
-            for (int w = 0; w < 8; ++w) tot += red[w];
+            for (int w = 0; w < 4; ++w) tot += red[w];
             *loss = tot / (float)B;
         }
     }
     if (t >= SPH_MLP_PARAMS) return;
-    float g = 0.0f;
-    for (int k = 0; k < splits; ++k) g += part[(size_t)k * SPH_MLP_PARAMS + t];
-    G[t] = g;
-    if (grads) grads[t] = g;
+    // four parameters a thread: every weight row, bias vector and layer starts
+    // at a multiple of four
+    static_assert(SPH_MLP_PARAMS % 4 == 0 && MLP_IN % 4 == 0, "whole quads");
+    auto at4 = [&](const float* p) { return *reinterpret_cast<const float4*>(p + t); };
+    float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int k = 0; k < splits; ++k) {
+        const float4 p = at4(part + (size_t)k * SPH_MLP_PARAMS);
+        g[0] += p.x;
+        g[1] += p.y;
+        g[2] += p.z;
+        g[3] += p.w;
+    }
+    *reinterpret_cast<float4*>(G + t) = make_float4(g[0], g[1], g[2], g[3]);
+    if (grads)
+        for (int e = 0; e < 4; ++e) grads[t + e] = g[e];  // the caller's array, of any alignment
     if (!adam) return;
-    // phase 0 leaves the error head (row 3 of W4, b4[3]), phase 1 trains it alone
-    const bool head = (t >= L.w[3] + 3 * MLP_H && t < L.w[3] + 4 * MLP_H) || t == L.b[3] + 3;
-    if (head != (o.phase == 1)) return;
-    const float m = o.b1 * Mo[t] + (1.f - o.b1) * g;
-    const float v = o.b2 * Vo[t] + (1.f - o.b2) * g * g;
-    Mo[t] = m;
-    Vo[t] = v;
-    const float p = P[t] - o.lr * (m / o.c1) / (sqrtf(v / o.c2) + o.eps);
-    P[t] = p;
     const int l = t >= L.w[3] ? 3 : (t >= L.w[2] ? 2 : (t >= L.w[1] ? 1 : 0));
-    const int e = t - L.w[l];
-    if (e < L.wn[l]) {
-        const __nv_bfloat16 w = __float2bfloat16_rn(p);
-        W[t] = w;
-        WT[L.w[l] + (e % L.in[l]) * L.out[l] + e / L.in[l]] = w;
+    const int e0 = t - L.w[l], nin = l == 0 ? MLP_IN : MLP_H, nout = l == 3 ? MLP_OUT : MLP_H;
+    const float4 P4 = at4(P), M4 = at4(Mo), V4 = at4(Vo);
+    float p[4] = {P4.x, P4.y, P4.z, P4.w}, m[4] = {M4.x, M4.y, M4.z, M4.w}, v[4] = {V4.x, V4.y, V4.z, V4.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        // phase 0 leaves the error head (row 3 of W4, b4[3]), phase 1 trains it alone
+        const bool head = (t >= L.w[3] + 3 * MLP_H && t < L.w[3] + 4 * MLP_H) || t + e == L.b[3] + 3;
+        if (head != (o.phase == 1)) continue;
+        m[e] = o.b1 * m[e] + (1.f - o.b1) * g[e];
+        v[e] = o.b2 * v[e] + (1.f - o.b2) * g[e] * g[e];
+        p[e] -= o.lr * (m[e] / o.c1) / (sqrtf(v[e] / o.c2) + o.eps);
+    }
+    *reinterpret_cast<float4*>(Mo + t) = make_float4(m[0], m[1], m[2], m[3]);
+    *reinterpret_cast<float4*>(Vo + t) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(P + t) = make_float4(p[0], p[1], p[2], p[3]);
+    if (e0 < nin * nout) {
+        const int r = e0 / nin, c = e0 % nin;
+        const __nv_bfloat162 lo2 = __floats2bfloat162_rn(p[0], p[1]), hi2 = __floats2bfloat162_rn(p[2], p[3]);
+        *reinterpret_cast<__nv_bfloat162*>(W + t) = lo2;
+        *reinterpret_cast<__nv_bfloat162*>(W + t + 2) = hi2;
+        __nv_bfloat16* wt = WT + L.w[l] + c * nout + r;
+        wt[0] = lo2.x;
+        wt[nout] = lo2.y;
+        wt[2 * nout] = hi2.x;
+        wt[3 * nout] = hi2.y;
     }
 }
 
@@ -1095,7 +1157,7 @@ struct sph_mlp {
     __nv_bfloat16 *DT[3], *DYT;        // transposed gradients of the pre-activations and of the output
     float* part;                       // split-K partials: `splits` packed parameter vectors
     int splits;
-    float* loss_part;                  // two partial losses per 32 rows
+    float* loss_part;                  // two partial losses per CTA of 16 rows or more
     float* loss;
     unsigned* err;
     long long step;
@@ -1162,7 +1224,7 @@ static size_t mlp_carve(sph_mlp* m, uintptr_t base)
     m->DYT = c.take<__nv_bfloat16>((size_t)MLP_OUT * B);
     m->splits = max_splits(m->max_batch);
     m->part = c.take<float>((size_t)m->splits * P);
-    m->loss_part = c.take<float>(2 * (B / 32));
+    m->loss_part = c.take<float>(2 * (B / 16));
     m->loss = c.take<float>(4);
     m->err = c.take<unsigned>(4);
     return (c.off + 255) & ~(uintptr_t)255;
@@ -1260,12 +1322,15 @@ static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const 
     a.dyt = m->DYT;
     a.loss_part = m->loss_part;
     a.err = m->err;
-    // 32 rows a CTA while one wave of CTAs takes the batch (its weights are
-    // streamed once per CTA), 64 beyond
-    const int NB = B <= 32 * sms ? 32 : 64;
+    // as few rows a CTA as one wave of CTAs allows: the epilogues (1.85 us a
+    // step per 32 rows, bound by the GELU's reciprocals and exponentials) are
+    // most of the chain
+    const int NB = B <= 16 * sms ? 16 : (B <= 32 * sms ? 32 : 64);
     CUtensorMap mx;
     MLP_TRY(m, make_map(&mx, x, B, MLP_IN, MLP_IN, NB));
-    rc = NB == 32 ? launch_rows<32>(m, mx, a, s) : launch_rows<64>(m, mx, a, s);
+    rc = NB == 16   ? launch_rows<16>(m, mx, a, s)
+         : NB == 32 ? launch_rows<32>(m, mx, a, s)
+                    : launch_rows<64>(m, mx, a, s);
     if (rc != SPH_OK) return rc;
     static bool attr = false;
     if (!attr) {
@@ -1280,7 +1345,7 @@ static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const 
     k_train_dw<<<dim3(dw::TILES - first, splits), 128, dw::TOTAL, s>>>(m->dmaps, first, kb, per, m->part, m->err);
     AdamArgs none;
     memset(&none, 0, sizeof(none));
-    k_train_update<<<(SPH_MLP_PARAMS - lo + 255) / 256, 256, 0, s>>>(
+    k_train_update<<<(SPH_MLP_PARAMS - lo + 511) / 512, 128, 0, s>>>(
         m->part, splits, lo, m->G, grads, adam != nullptr, adam ? *adam : none, m->P, m->Mo, m->Vo, m->W, m->WT,
         m->loss_part, 2 * (B / NB), B, loss);
     m->launches += 2;

@@ -24,9 +24,10 @@ def _network(seed):
 
 
 # 128: one slice per 64 rows; 320 -> 384: uneven slices; 1152: all eight
-# slices; 32 rows per CTA up to 32 x the multiprocessors, 64 beyond; a handle
+# slices; 16, 32, 64 rows per CTA up to 16 and 32 x the multiprocessors and
+# beyond; a handle
 # made for more rows than the batch (longer transposed rows)
-@pytest.mark.parametrize("B,max_batch", [(128, 128), (384, 384), (384, 2048), (1152, 1152), (4864, 4992),
+@pytest.mark.parametrize("B,max_batch", [(128, 128), (384, 384), (384, 2048), (1152, 1152), (2432, 2432), (2560, 2560), (4864, 4992),
                                          (4992, 4992), (9984, 9984)])
 def test_gradients_at_batch_edges(B, max_batch):
     p, packed = _network(61)
@@ -48,7 +49,7 @@ def test_gradients_at_batch_edges(B, max_batch):
             assert np.linalg.norm(a - r) <= 7 * 2.0 ** -9 * np.linalg.norm(r), (name, np.linalg.norm(a - r) / np.linalg.norm(r))
 
 
-@pytest.mark.parametrize("B", [128, 640, 5120])
+@pytest.mark.parametrize("B", [128, 640, 3072, 5120])
 def test_loss_and_phases_at_batch_edges(B):
     """The loss of both phases against the oracle's, and what each phase
     leaves alone; the same step from the same state gives the same bits."""

@@ -49,11 +49,43 @@ struct GemmEpi {
 // approximations, which add a few 1e-7: far below the BF16 rounding of the
 // activations (2^-9 relative).  The GELU epilogue bounds the fused forward
 // pass; this form takes about half the instructions of the library erff.
-//
-// Two values at a time with the packed FP32x2 instructions: exp(-z^2 / 2) =
-// 2^(-z^2 log2(e) / 2) on the hardware base-2 exponential and Phi(z) = 1/2 +
-// sign(z) (1/2 - Phi(-|z|)), the sign bit of z moved onto the bracket, so
-// that each step but the reciprocal and the exponential works on both.
+// Also returns exp(-z^2 / 2) for the derivative.
+__device__ __forceinline__ float phi_lower(float z, float* gauss)
+{
+    const float az = fabsf(z);
+    const float t = __fdividef(1.0f, fmaf(0.23164190f, az, 1.0f));  // p / sqrt 2 = 0.3275911 / 1.41421356
+    float poly = fmaf(t, 0.5307027145f, -0.7265760135f);            // a_k / 2
+    poly = fmaf(t, poly, 0.7107068705f);
+    poly = fmaf(t, poly, -0.142248368f);
+    poly = fmaf(t, poly, 0.127414796f);
+    poly *= t;
+    const float e = __expf(-0.5f * z * z);
+    *gauss = e;
+    return poly * e;
+}
+
+// GELU(z) = z Phi(z) and its derivative Phi(z) + z phi(z), phi the standard
+// normal density, with Phi(z) = 1 - Phi(-z) for z >= 0.
+__device__ __forceinline__ float gelu_f(float z)
+{
+    float e;
+    const float lt = phi_lower(z, &e);
+    return z * (z >= 0.0f ? 1.0f - lt : lt);
+}
+
+__device__ __forceinline__ float gelu_grad_f(float z)
+{
+    float e;
+    const float lt = phi_lower(z, &e);
+    return (z >= 0.0f ? 1.0f - lt : lt) + z * e * 0.39894228040143268f;
+}
+
+// GELU of two values with the packed FP32x2 instructions (the fused
+// forward's epilogue): the same formula as gelu_f, with
+// exp(-z^2 / 2) = 2^(-z^2 log2(e) / 2) on the hardware base-2 exponential
+// and Phi(z) = 1/2 + sign(z) (1/2 - Phi(-|z|)), the sign bit of z moved onto
+// the bracket, so that each step but the reciprocal and the exponential
+// works on both values at once.
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -61,49 +93,35 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
-// Phi(z); gauss = exp(-z^2 / 2).
-__device__ __forceinline__ float2 phi2_f(float2 z, float2& gauss)
+__device__ __forceinline__ float2 gelu2_f(float2 z)
 {
     const float2 az = make_float2(fabsf(z.x), fabsf(z.y));
-    const float2 d = __ffma2_rn(make_float2(0.23164190f, 0.23164190f), az, make_float2(1.0f, 1.0f));  // p / sqrt 2
+    const float2 d = __ffma2_rn(make_float2(0.23164190f, 0.23164190f), az, make_float2(1.0f, 1.0f));
     const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
     float2 poly = __ffma2_rn(t, make_float2(0.5307027145f, 0.5307027145f), make_float2(-0.7265760135f, -0.7265760135f));
-    poly = __ffma2_rn(t, poly, make_float2(0.7107068705f, 0.7107068705f));  // a_k / 2
+    poly = __ffma2_rn(t, poly, make_float2(0.7107068705f, 0.7107068705f));
     poly = __ffma2_rn(t, poly, make_float2(-0.142248368f, -0.142248368f));
     poly = __ffma2_rn(t, poly, make_float2(0.127414796f, 0.127414796f));
     poly = __fmul2_rn(poly, t);
     // -z^2 log2(e) / 2
     const float2 a = __fmul2_rn(__fmul2_rn(z, make_float2(-0.72134752f, -0.72134752f)), z);
-    gauss = make_float2(ex2_approx(a.x), ex2_approx(a.y));
-    const float2 lt = __fmul2_rn(poly, gauss);                                              // Phi(-|z|)
+    const float2 e = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+    const float2 lt = __fmul2_rn(poly, e);                                              // Phi(-|z|)
     const float2 hb = __ffma2_rn(lt, make_float2(-1.0f, -1.0f), make_float2(0.5f, 0.5f));  // 1/2 - Phi(-|z|)
     const float2 sh = make_float2(__uint_as_float(__float_as_uint(hb.x) ^ (__float_as_uint(z.x) & 0x80000000u)),
                                   __uint_as_float(__float_as_uint(hb.y) ^ (__float_as_uint(z.y) & 0x80000000u)));
-    return __fadd2_rn(sh, make_float2(0.5f, 0.5f));
-}
-
-// GELU(z) = z Phi(z).
-__device__ __forceinline__ float2 gelu2_f(float2 z)
-{
-    float2 gauss;
-    const float2 phi = phi2_f(z, gauss);
-    return __fmul2_rn(z, phi);
-}
-
-// GELU'(z) = Phi(z) + z phi(z), phi the standard normal density.
-__device__ __forceinline__ float2 gelu_grad2_f(float2 z)
-{
-    float2 gauss;
-    const float2 phi = phi2_f(z, gauss);
-    return __ffma2_rn(__fmul2_rn(z, gauss), make_float2(0.39894228040143268f, 0.39894228040143268f), phi);
+    return __fmul2_rn(z, __fadd2_rn(sh, make_float2(0.5f, 0.5f)));
 }
 
 __global__ void k_debug_gelu(const float* __restrict__ z, int n, int grad, float* __restrict__ out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float2 zz = make_float2(z[i], 0.0f);
-    out[i] = grad == 1 ? gelu_grad2_f(zz).x : gelu2_f(zz).x;
+    if (grad == 2) {
+        out[i] = gelu2_f(make_float2(z[i], 0.0f)).x;
+        return;
+    }
+    out[i] = grad ? gelu_grad_f(z[i]) : gelu_f(z[i]);
 }
 
 // Epilogue, in column chunks of EC (32, or NT when NT < 32), through shared
@@ -893,9 +911,10 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
                     uint32_t(&p)[CH / 2] = pk[c / CH];
 #pragma unroll
                     for (int e = 0; e < CH; e += 2) {
-                        const float2 zz = __fadd2_rn(make_float2(z[e], z[e + 1]), make_float2(b, b));
-                        const float2 r = s < 3 ? gelu2_f(zz) : __fmul2_rn(make_float2(v[e], v[e + 1]), gelu_grad2_f(zz));
-                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(r.x, r.y);
+                        const float z0 = z[e] + b, z1 = z[e + 1] + b;
+                        const __nv_bfloat162 h2 =
+                            s < 3 ? __floats2bfloat162_rn(gelu_f(z0), gelu_f(z1))
+                                  : __floats2bfloat162_rn(v[e] * gelu_grad_f(z0), v[e + 1] * gelu_grad_f(z1));
                         p[e >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
                     }
                     if (s < 6) {  // the next step's operand: (row n0 + c + e, feature f)
@@ -933,18 +952,22 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
 // Weight and bias gradients of every layer: dW[out][in] = dT[out][B] .
 // inT[in][B]^T over a slice of the batch.  blockIdx.x: a tile of 128 outputs
 // x 144 inputs of a layer (two N tiles cover 256 or 272 inputs: 14 tiles in
-// all), blockIdx.y: the slice.  The first N tile also sums dT over its
-// batch rows, the bias gradient, as a product with a tile of ones (16 more
-// accumulator columns).  Partials go to part[slice] in the packed parameter
-// layout.  One kernel for all layers: a product alone would use 16 SMs.
+// all), blockIdx.y: the slice.  Partials go to part[slice] in the packed
+// parameter layout.  One kernel for all layers: a product alone would use
+// 16 SMs.  The last blocks of the first slice sum dT over the batch, the
+// bias gradients: a thread per output adds its row in batch order, one
+// float32 sum (its last bit reaches the next step's activations, so the
+// order is part of the result).  The rows come through the same TMA ring
+// (read straight from memory, a warp's loads of 32 rows were 32 wavefronts
+// each: 21 us for 2,048 rows), so that the chain of additions, 4 cycles
+// each, is what it takes.
 namespace dw {
-constexpr int NT = 144, STAGES = 4, TILES = 14;
+constexpr int NT = 144, STAGES = 4, TILES = 14, BIAS = 7;  // weight tiles, blocks of 128 biases
 constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = NT * BK * 2, STAGE = A_BYTES + B_BYTES;
-constexpr uint32_t ONES = STAGES * STAGE, ONES_BYTES = 16 * BK * 2;
-constexpr uint32_t BARS = ONES + ONES_BYTES;
+constexpr uint32_t BARS = STAGES * STAGE;
 constexpr uint32_t TOTAL = 1024 + BARS + 8 * (2 * STAGES + 1) + 16;
 constexpr uint32_t TMEM_COLS = 256;
-static_assert(STAGE % 1024 == 0 && ONES_BYTES % 1024 == 0, "operand tiles start on 1024-byte boundaries");
+static_assert(STAGE % 1024 == 0, "operand tiles start on 1024-byte boundaries");
 }  // namespace dw
 
 struct DwMaps {
@@ -952,11 +975,14 @@ struct DwMaps {
     CUtensorMap in[4];  // inT of layers 0 .. 3, boxes of 144 rows
 };
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(160)
 k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, int kb_per_split,
            float* __restrict__ part, unsigned* __restrict__ err)
 {
     using namespace dw;
+    const int tile = first_tile + (int)blockIdx.x;
+    const bool bias = tile >= TILES;
+    if (bias && blockIdx.y) return;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -967,23 +993,75 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
     const uint32_t done = bars + 8u * (2 * STAGES), tmem_slot = done + 8u;
     uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(gbase + BARS + 8 * (2 * STAGES + 1));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tile = first_tile + (int)blockIdx.x;
-    const int l = tile < 12 ? tile >> 2 : 3, mt = tile < 12 ? (tile >> 1) & 1 : 0, nt = tile & 1;
-    const int m0 = mt * BM, n0 = nt * NT;
-    const int kb0 = blockIdx.y * kb_per_split, nk = min(kb_per_split, kb_total - kb0);
     const ParamLayout L;
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full(s), 1);
-            mbar_init(empty(s), 1);
+            mbar_init(empty(s), bias ? 128 : 1);
         }
         mbar_init(done, 1);
         mbar_fence_init();
     }
-    for (int e = threadIdx.x; e < (int)ONES_BYTES / 4; e += 128)
-        reinterpret_cast<uint32_t*>(gbase + ONES)[e] = 0x3f803f80u;  // BF16 ones (any swizzle is the same)
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (bias) {
+        // blocks 0 .. 5: halves of the hidden layers, 6: the output layer (the
+        // last block, also where it is the only one)
+        const int blk = BIAS - ((int)gridDim.x - (int)blockIdx.x), l = blk >> 1, m0 = (blk & 1) * BM;
+        __syncthreads();
+        if (warp == 4) {  // the copies' own warp: in a summing warp they would hold up its chain
+            if (lane == 0) {
+                int i = 0;
+                for (; i < kb_total; ++i) {
+                    const int st = i % STAGES;
+                    if (i >= STAGES && !mbar_wait(empty(st), (uint32_t)((i / STAGES) - 1) & 1u, err)) break;
+                    mbar_expect_tx(full(st), A_BYTES);
+                    tma_load_2d(&maps.d[l], full(st), base + st * STAGE, i * BK, m0);
+                }
+                if (i < kb_total)  // let the copies in flight land before the CTA goes away
+                    for (int q = max(0, i - STAGES); q < i; ++q)
+                        mbar_wait(full(q % STAGES), (uint32_t)(q / STAGES) & 1u, err);
+            }
+            return;
+        }
+        // a row's 64 values of a block are loaded while the block before is added
+        uint4 v[2][BK / 8];
+        float s = 0.f;
+        auto fetch = [&](int i, uint4 (&to)[BK / 8]) {
+            const int st = i % STAGES;
+            if (!mbar_wait(full(st), (uint32_t)(i / STAGES) & 1u, err)) return false;
+            const uint8_t* row = gbase + st * STAGE;
+#pragma unroll
+            for (int c = 0; c < BK / 8; ++c)
+                to[c] = *reinterpret_cast<const uint4*>(row + sw128_offset((int)threadIdx.x, 8 * c));
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty(st)) : "memory");
+            return true;
+        };
+        auto sum = [&](const uint4 (&from)[BK / 8]) {
+#pragma unroll
+            for (int c = 0; c < BK / 8; ++c) {
+                const uint32_t w[4] = {from[c].x, from[c].y, from[c].z, from[c].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {  // BF16 -> FP32 is the high half of the word
+                    s = __fadd_rn(s, __uint_as_float(w[j] << 16));
+                    s = __fadd_rn(s, __uint_as_float(w[j] & 0xffff0000u));
+                }
+            }
+        };
+        bool ok = fetch(0, v[0]);
+        for (int i = 0; ok && i < kb_total; i += 2) {  // an even number of blocks
+            ok = fetch(i + 1, v[1]);
+            sum(v[0]);
+            if (ok && i + 2 < kb_total) ok = fetch(i + 2, v[0]);
+            sum(v[1]);
+        }
+        const int f = m0 + (int)threadIdx.x;
+        if (ok && f < L.out[l])  // the other slices hold zeros
+            for (int k = 0; k < (int)gridDim.y; ++k) part[(size_t)k * SPH_MLP_PARAMS + L.b[l] + f] = k ? 0.0f : s;
+        return;
+    }
+    const int l = tile < 12 ? tile >> 2 : 3, mt = tile < 12 ? (tile >> 1) & 1 : 0, nt = tile & 1;
+    const int m0 = mt * BM, n0 = nt * NT;
+    const int kb0 = blockIdx.y * kb_per_split, nk = min(kb_per_split, kb_total - kb0);
+
     if (warp == 0) tmem_alloc(tmem_slot, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
@@ -1008,26 +1086,23 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
             for (int i = max(0, issued - STAGES); i < issued; ++i)
                 mbar_wait(full(i % STAGES), (uint32_t)(i / STAGES) & 1u, err);
     } else if (warp == 1 && lane == 0) {
-        constexpr uint32_t idesc = umma_idesc_bf16(BM, NT), idesc1 = umma_idesc_bf16(BM, 16);
+        constexpr uint32_t idesc = umma_idesc_bf16(BM, NT);
         for (int i = 0; i < nk; ++i) {
             const int s = i % STAGES;
             if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, err)) break;
             tc_fence_after();
             const uint32_t a = base + s * STAGE, b = a + A_BYTES;
 #pragma unroll
-            for (int k = 0; k < BK / UK; ++k) {
+            for (int k = 0; k < BK / UK; ++k)
                 umma_bf16(tmem, sw128_desc(a + k * UK * 2), sw128_desc(b + k * UK * 2), idesc, (uint32_t)((i | k) != 0));
-                if (nt == 0)
-                    umma_bf16(tmem + NT, sw128_desc(a + k * UK * 2), sw128_desc(base + ONES + k * UK * 2), idesc1,
-                              (uint32_t)((i | k) != 0));
-            }
             umma_commit(empty(s));
         }
         umma_commit(done);
     }
     __syncwarp();
 
-    const bool ok = mbar_wait(done, 0, err);
+    // warps 0 .. 3 each read their tensor-memory lanes
+    const bool ok = warp < 4 && mbar_wait(done, 0, err);
     tc_fence_after();
     if (ok) {
         const int m = m0 + warp * 32 + lane, nin = L.in[l];
@@ -1053,11 +1128,6 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
                          "r"(smem_u32(stage)), "r"(w * 4)
                          : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
-        if (nt == 0) {
-            float v[16];
-            tmem_ld16(row + NT, v);
-            if (m < L.out[l]) out[L.b[l] + m] = v[0];
         }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -1123,8 +1193,10 @@ k_train_update(const float* __restrict__ part, int splits, int lo, float* __rest
         // phase 0 leaves the error head (row 3 of W4, b4[3]), phase 1 trains it alone
         const bool head = (t >= L.w[3] + 3 * MLP_H && t < L.w[3] + 4 * MLP_H) || t + e == L.b[3] + 3;
         if (head != (o.phase == 1)) continue;
-        m[e] = o.b1 * m[e] + (1.f - o.b1) * g[e];
-        v[e] = o.b2 * v[e] + (1.f - o.b2) * g[e] * g[e];
+        // contracted in one fixed way: a last bit here decides now and then how
+        // a weight rounds to BF16
+        m[e] = __fmaf_rn(1.f - o.b1, g[e], __fmul_rn(o.b1, m[e]));
+        v[e] = __fmaf_rn(__fmul_rn(1.f - o.b2, g[e]), g[e], __fmul_rn(o.b2, v[e]));
         p[e] -= o.lr * (m[e] / o.c1) / (sqrtf(v[e] / o.c2) + o.eps);
     }
     *reinterpret_cast<float4*>(Mo + t) = make_float4(m[0], m[1], m[2], m[3]);
@@ -1342,7 +1414,8 @@ static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const 
     const int per = (kb + splits - 1) / splits;
     splits = (kb + per - 1) / per;
     const int first = phase == 0 ? 0 : 12, lo = phase == 0 ? 0 : L.w[3];
-    k_train_dw<<<dim3(dw::TILES - first, splits), 128, dw::TOTAL, s>>>(m->dmaps, first, kb, per, m->part, m->err);
+    const int nbias = phase == 0 ? dw::BIAS : 1;
+    k_train_dw<<<dim3(dw::TILES - first + nbias, splits), 160, dw::TOTAL, s>>>(m->dmaps, first, kb, per, m->part, m->err);
     AdamArgs none;
     memset(&none, 0, sizeof(none));
     k_train_update<<<(SPH_MLP_PARAMS - lo + 511) / 512, 128, 0, s>>>(

@@ -191,54 +191,101 @@ k_density(const float4* __restrict__ pos, const float4* __restrict__ vel, SoaPos
 }
 
 
-// Only the slots of a list whose length the device holds (the list is built
-// on the device; warps stride over it): a warp per particle, the lanes fetch
-// the walk's rows together and test a row's candidates side by side, then
-// the hits are added in slot order by the same fused multiply-adds as the
-// one-thread pass (the lanes pass the terms by shuffles), so the density is
-// bit for bit the full pass's.  Kept for few particles (the exact-local
-// path), where the one-thread walk leaves its latency exposed.
-__global__ void __launch_bounds__(256)
-k_density_list(const float4* __restrict__ pos, const unsigned* __restrict__ start, Scenes sc,
-               float* __restrict__ rho, float2* __restrict__ ab, int* __restrict__ nbr, int* __restrict__ ncand,
+// A warp per particle, for launches too small to fill the chip with a thread
+// per particle, where a thread's serial walk of some 25 rows leaves its
+// latency exposed, and for lists of few particles (LIST: the slots
+// list[0 .. *list_len), built on the device).  The lanes fetch the walk's rows
+// together, cut them into pieces of at most 32 slots (a segment each) and
+// test the pieces' candidates side by side by flat index; the hits are added
+// in walk order by the same fused multiply-adds as the one-thread pass (the
+// lanes pass the terms by shuffles), and the lane of a piece gathers its
+// mask from the rounds' ballots.  Same bits as density_at.  Bound by latency:
+// 4,112 particles take 12 us where the one-thread pass takes 42 (16 blocks,
+// each thread some 100 candidates in series).
+template <bool SEG, bool LIST>
+__global__ void __launch_bounds__(128)
+k_density_warp(const float4* __restrict__ pos, const float4* __restrict__ vel, const unsigned* __restrict__ start,
+               Scenes sc, float* __restrict__ rho, float2* __restrict__ ab, float4* __restrict__ prec,
+               int* __restrict__ nbr, uint2* __restrict__ seg, int* __restrict__ nseg, int* __restrict__ ncand,
                const int* __restrict__ list, const unsigned* __restrict__ list_len, unsigned* __restrict__ err)
 {
     const int lane = threadIdx.x & 31;
     const int nw = gridDim.x * (blockDim.x >> 5);
-    const int len = (int)min(*list_len, (unsigned)sc.n_all);
+    const int len = LIST ? (int)min(*list_len, (unsigned)sc.n_all) : sc.n_all;
     for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < len; w += nw) {
-        const int i = list[w];
+        const int i = LIST ? list[w] : w;
         const StepConst& c = sc.c[scene_of(sc.pbase, sc.S, (unsigned)i)];
         const float h2 = c.h2;
         const int nb_all = sc.nb_all;
         const float4 pi = pos[i];
         const bool att_i = id_of(pi) < nb_all;
         float sum = 0.0f;
-        int cnt = 0, nc = 0;
+        int cnt = 0, nc = 0, ns = 0;
         WarpRows rows(c.g, c.wg, start + c.c_base, pi.x, pi.y, pi.z);
         for (int bt = 0; 32 * bt < rows.nrows; ++bt) {
             rows.batch(bt);
-            const unsigned total = rows.flatten();
-            nc += (int)total;
-            for (unsigned k0 = 0; k0 < total; k0 += 32) {
-                const unsigned k = k0 + (unsigned)lane;
-                const unsigned j = rows.slot(k < total ? k : total - 1);
-                bool hit = false, self = false;
-                float t = 0.0f;
-                if (k < total) {
-                    const float4 pj = __ldg(pos + j);
-                    const float r2 = pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z));
-                    self = j == (unsigned)i;
-                    hit = r2 < h2 && !(att_i && !self && id_of(pj) < nb_all);
-                    t = h2 - r2;
+            if (rows.s0 < rows.s1 && !SPH_IN_BOUNDS(rows.s1 - 1u, sc.n_all, err)) rows.s1 = rows.s0;
+            const unsigned r0 = rows.s0, r1 = rows.s1;
+            const unsigned np = (r1 - r0 + 31u) >> 5;  // pieces of this lane's row
+            const bool one = !__any_sync(FULL, np > 1u);
+            unsigned pinc = np;
+            if (!one)
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned u = __shfl_up_sync(FULL, pinc, o);
+                    if (lane >= o) pinc += u;
                 }
-                unsigned m = __ballot_sync(FULL, hit);
-                cnt += __popc(m & ~__ballot_sync(FULL, self));
-                while (m) {  // the hits in walk order, one fused multiply-add each
-                    const int q = __ffs(m) - 1;
-                    m &= m - 1u;
-                    const float v = __shfl_sync(FULL, t, q);
-                    sum = fmaf(v * v, v, sum);
+            const unsigned pieces = one ? 32u : __shfl_sync(FULL, pinc, 31);
+            for (unsigned p0 = 0; p0 < pieces; p0 += 32) {
+                if (!one) {  // this lane's piece p0 + lane: the row whose pieces hold it
+                    const unsigned p = p0 + (unsigned)lane;
+                    int lo = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)  // rows before it: those whose last piece is <= p
+                        if (__shfl_sync(FULL, pinc, lo + step - 1) <= p) lo += step;
+                    const unsigned a = __shfl_sync(FULL, r0, lo), e = __shfl_sync(FULL, r1, lo);
+                    const unsigned k = p - (__shfl_sync(FULL, pinc, lo) - __shfl_sync(FULL, np, lo));
+                    rows.s0 = rows.s1 = 0;
+                    if (p < pieces) {
+                        rows.s0 = a + 32u * k;
+                        rows.s1 = min(rows.s0 + 32u, e);
+                    }
+                }
+                const unsigned total = rows.flatten();
+                nc += (int)total;
+                unsigned mine = 0;  // hits of this lane's piece, bit = slot - its first
+                for (unsigned k0 = 0; k0 < total; k0 += 32) {
+                    const unsigned k = k0 + (unsigned)lane;
+                    const unsigned j = rows.slot(k < total ? k : total - 1);
+                    bool hit = false, self = false;
+                    float t = 0.0f;
+                    if (k < total) {
+                        const float4 pj = __ldg(pos + j);
+                        const float r2 = pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z));
+                        self = j == (unsigned)i;
+                        hit = r2 < h2 && !(att_i && !self && id_of(pj) < nb_all);
+                        t = h2 - r2;
+                    }
+                    unsigned m = __ballot_sync(FULL, hit);
+                    cnt += __popc(att_i ? m & ~__ballot_sync(FULL, self) : m);
+                    if (SEG) {
+                        const int o = (int)(k0 - rows.pre);  // flat index of the round less the piece's
+                        const unsigned in = o >= 0 ? (o < 32 ? m << o : 0u) : (o > -32 ? m >> -o : 0u);
+                        const unsigned plen = rows.s1 - rows.s0;
+                        mine |= in & (plen < 32u ? (1u << plen) - 1u : FULL);
+                    }
+                    const float tt = __fmul_rn(t, t);
+                    while (m) {  // the hits in walk order, one fused multiply-add each
+                        const int q = __ffs((int)m) - 1;
+                        m &= m - 1u;
+                        sum = fmaf(__shfl_sync(FULL, tt, q), __shfl_sync(FULL, t, q), sum);
+                    }
+                }
+                if (SEG && !att_i) {
+                    const unsigned has = __ballot_sync(FULL, mine != 0u);
+                    const int k = ns + __popc(has & ((1u << lane) - 1u));
+                    if (mine && k < SEG_CAP) seg[(size_t)i * SEG_CAP + k] = make_uint2(rows.s0, mine);
+                    ns += __popc(has);
                 }
             }
         }
@@ -246,12 +293,28 @@ k_density_list(const float4* __restrict__ pos, const unsigned* __restrict__ star
             ncand[i] = nc;
             const float r = c.mC6 * sum;
             rho[i] = r;
-            ab[i] = make_float2(c.mass / r, c.k * (r - c.rho0));
-            nbr[i] = cnt;
+            const float2 abi = make_float2(c.mass / r, c.k * (r - c.rho0));
+            ab[i] = abi;
+            if (prec) {
+                const float4 v = __ldg(vel + i);
+                prec[2 * i] = make_float4(pi.x, pi.y, pi.z, abi.y);
+                prec[2 * i + 1] = make_float4(v.x, v.y, v.z, att_i ? -abi.x : abi.x);
+            }
+            nbr[i] = att_i ? cnt : cnt - 1;  // less the particle itself
+            if (SEG) nseg[i] = ns;
             if (!isfinite(r)) atomicOr(err, SPH_DEV_NONFINITE);
         }
     }
 }
+
+// The density pass takes a warp per particle up to this many particles per
+// multiprocessor (16,416 on 152), a thread per particle beyond.  Whole step
+// replayed, us, thread / warp: dam-break of 2,000 particles at spacing h/2
+// 68 / 42, 16,000 73 / 57, 33,000 79 / 74, 66,000 81 / 106; at about 100
+// neighbours and h cells 16,000 106 / 105, 24,000 106 / 124; compressed
+// fluid of about 250 neighbours 16,000 183 / 154, 33,000 218 / 225.
+constexpr int DENSITY_WARP_PER_SM = 108;
+constexpr int WARP_BLOCKS = 64;  // blocks of four warps per multiprocessor, at most
 
 cudaError_t launch_density(const float4* pos, const float4* vel, const SoaPos& xyz, const unsigned* start,
                            const Scenes& sc, const Tuning& t, float* rho, float2* ab, float4* prec, int* nbr,
@@ -259,17 +322,28 @@ cudaError_t launch_density(const float4* pos, const float4* vel, const SoaPos& x
                            unsigned* err, cudaStream_t s, long long* launches)
 {
     if (sc.n_all <= 0) return cudaSuccess;
-    const int per_block = t.block * (t.ppt > 1 ? t.ppt : 1);
-    const int all = (sc.n_all + per_block - 1) / per_block;
+    const bool use_seg = seg && t.use_seg;
+    // blocks of a warp per particle; they stride over the particles
+    const int cap = WARP_BLOCKS * sm_count();
+    const int wblocks = (sc.n_all + 3) / 4 < cap ? (sc.n_all + 3) / 4 : cap;
     if (list) {
-        const int cap = 16 * sm_count();  // 8 warps per block, 16 blocks per SM at most
-        const int blocks = (sc.n_all + 7) / 8 < cap ? (sc.n_all + 7) / 8 : cap;
-        k_density_list<<<blocks, 256, 0, s>>>(pos, start, sc, rho, ab, nbr, ncand, list, list_len, err);
-    } else if (seg && t.use_seg) {
-        k_density<true><<<all, t.block, 0, s>>>(pos, vel, xyz, start, sc, rho, ab, prec, nbr, seg, nseg, ncand, err);
+        k_density_warp<false, true><<<wblocks, 128, 0, s>>>(pos, vel, start, sc, rho, ab, prec, nbr, nullptr, nullptr,
+                                                            ncand, list, list_len, err);
+    } else if (sc.n_all <= DENSITY_WARP_PER_SM * sm_count()) {
+        if (use_seg)
+            k_density_warp<true, false><<<wblocks, 128, 0, s>>>(pos, vel, start, sc, rho, ab, prec, nbr, seg, nseg,
+                                                                ncand, nullptr, nullptr, err);
+        else
+            k_density_warp<false, false><<<wblocks, 128, 0, s>>>(pos, vel, start, sc, rho, ab, prec, nbr, nullptr,
+                                                                 nullptr, ncand, nullptr, nullptr, err);
     } else {
-        k_density<false><<<all, t.block, 0, s>>>(pos, vel, xyz, start, sc, rho, ab, prec, nbr, seg, nseg, ncand,
-                                                 err);
+        const int per_block = t.block * (t.ppt > 1 ? t.ppt : 1);
+        const int all = (sc.n_all + per_block - 1) / per_block;
+        if (use_seg)
+            k_density<true><<<all, t.block, 0, s>>>(pos, vel, xyz, start, sc, rho, ab, prec, nbr, seg, nseg, ncand, err);
+        else
+            k_density<false><<<all, t.block, 0, s>>>(pos, vel, xyz, start, sc, rho, ab, prec, nbr, seg, nseg, ncand,
+                                                     err);
     }
     ++*launches;
     return cudaGetLastError();

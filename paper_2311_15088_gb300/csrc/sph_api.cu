@@ -35,8 +35,6 @@ struct sph_handle {
     int* tmp;
     int* tmp_id;              // ids beside tmp (the per-cell sort's ranking keys)
     unsigned *count, *cell_start, *scan_part;
-    int* big_list;
-    unsigned* big_count;
     float* rho;
     float2* ab;  // (m / rho, p) per sorted slot
     int* nbr;
@@ -54,8 +52,6 @@ struct sph_handle {
     unsigned *bkey, *brank;
     int* btmp;
     unsigned *bcount, *bstart, *bscan_part;
-    int* bbig_list;
-    unsigned* bbig_count;
     float4* fb;
     float4* obst;             // obstacle grid over the boid grid (nbcells)
     float* obst_shapes;       // spheres then boxes (SPH_MAX_OBSTACLES x 10 floats)
@@ -350,8 +346,6 @@ static size_t carve(sph_handle* h, uintptr_t base)
     h->count = cv.take<unsigned>(C);
     h->cell_start = cv.take<unsigned>(C + 1);
     h->scan_part = cv.take<unsigned>((size_t)scan_parts((int)C) + 1);
-    h->big_list = cv.take<int>(C);
-    h->big_count = cv.take<unsigned>(1);
     h->rho = cv.take<float>(n);
     h->ab = cv.take<float2>(n);
     h->nbr = cv.take<int>(n);
@@ -375,8 +369,6 @@ static size_t carve(sph_handle* h, uintptr_t base)
     h->bcount = cv.take<unsigned>(Cb);
     h->bstart = cv.take<unsigned>(Cb + 1);
     h->bscan_part = cv.take<unsigned>((size_t)scan_parts((int)Cb) + 1);
-    h->bbig_list = cv.take<int>(Cb);
-    h->bbig_count = cv.take<unsigned>(1);
     h->fb = cv.take<float4>(nb);
     h->obst = cv.take<float4>(Cb);
     h->obst_shapes = cv.take<float>((size_t)SPH_MAX_OBSTACLES * 10);
@@ -630,7 +622,6 @@ int sph_batch_create(const sph_params* params, const int* n_fluid, const int* n_
     if (e == cudaSuccess) e = cudaMemcpy(h->d_pbase, h->h_pbase, sizeof(unsigned) * (size_t)(S + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_bbase, h->h_bbase, sizeof(unsigned) * (size_t)(S + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(h->err, 0, 4 * sizeof(unsigned));
-    if (e == cudaSuccess) e = prepare_kernels();
     if (e == cudaSuccess && h->n_boid > 0) {
         // default priority: a higher one lets the F_b warps take SMs from the
         // fluid blocks early and slows the force pass by more than it saves
@@ -904,8 +895,8 @@ static SoaPos soa_of(const sph_handle* h)
 }
 
 // Keys (if needed), scan, scatter and per-cell sort + gather of the state
-// into the sorted scratch arrays.  consume = true zeroes the counts for the
-// next step's keys.
+// into the sorted scratch arrays.  consume = true zeroes the counts (in the
+// scan) for the next step's keys.
 static int bin_state(sph_handle* h, cudaStream_t s, bool consume)
 {
     if (!h->keys_ready) {
@@ -916,21 +907,17 @@ static int bin_state(sph_handle* h, cudaStream_t s, bool consume)
         h->keys_ready = true;
     }
     prof_begin(h, SPH_KIND_SCAN, s);
-    CUDA_TRY(h, launch_scan(h->count, h->ncells, h->scan_part, h->cell_start, s, &h->launches));
+    CUDA_TRY(h, launch_scan(h->count, h->ncells, h->scan_part, h->cell_start, consume, s, &h->launches));
     prof_end(h, s);
     prof_begin(h, SPH_KIND_SCATTER, s);
     CUDA_TRY(h, launch_scatter_ids(h->key, h->rank, h->cell_start, h->pos, h->n, h->tmp, h->tmp_id, s,
                                    &h->launches));
     prof_end(h, s);
     prof_begin(h, SPH_KIND_SORT, s);
-    CUDA_TRY(h, launch_cellsort_slots(h->cell_start, h->key, h->n, h->ncells, h->tmp, h->tmp_id, h->pos, h->vel,
-                                      h->pos_s, h->vel_s, h->soa, h->n_boid, h->slot_of_boid, h->big_list,
-                                      h->big_count, s, &h->launches));
+    CUDA_TRY(h, launch_cellsort_slots(h->cell_start, h->key, h->n, h->tmp, h->tmp_id, h->pos, h->vel, h->pos_s,
+                                      h->vel_s, h->soa, h->n_boid, h->slot_of_boid, s, &h->launches));
     prof_end(h, s);
-    if (consume) {
-        CUDA_TRY(h, cudaMemsetAsync(h->count, 0, (size_t)h->ncells * sizeof(unsigned), s));
-        h->keys_ready = false;
-    }
+    if (consume) h->keys_ready = false;
     return SPH_OK;
 }
 
@@ -940,10 +927,11 @@ static int enqueue_boid_bin(sph_handle* h, cudaStream_t s)
     prof_begin(h, SPH_KIND_BOID_BIN, s);
     CUDA_TRY(h, cudaMemsetAsync(h->bcount, 0, (size_t)h->nbcells * sizeof(unsigned), s));
     CUDA_TRY(h, launch_boid_keys(h->bpos, h->sc, h->bkey, h->brank, h->bcount, s, &h->launches));
-    CUDA_TRY(h, launch_scan(h->bcount, h->nbcells, h->bscan_part, h->bstart, s, &h->launches));
+    CUDA_TRY(h, launch_scan(h->bcount, h->nbcells, h->bscan_part, h->bstart, false, s, &h->launches));
     CUDA_TRY(h, launch_scatter(h->bkey, h->brank, h->bstart, h->n_boid, h->btmp, s, &h->launches));
-    CUDA_TRY(h, launch_cellsort_gather(h->bstart, h->nbcells, h->btmp, h->bpos, h->bvel, h->bpos_s, h->bvel_s, 0,
-                                       nullptr, h->bbig_list, h->bbig_count, s, &h->launches));
+    // a boid's storage index is its id
+    CUDA_TRY(h, launch_cellsort_slots(h->bstart, h->bkey, h->n_boid, h->btmp, h->btmp, h->bpos, h->bvel, h->bpos_s,
+                                      h->bvel_s, nullptr, 0, nullptr, s, &h->launches));
     prof_end(h, s);
     return SPH_OK;
 }
@@ -970,7 +958,7 @@ static int enqueue_neighbor_passes(sph_handle* h, cudaStream_t s, bool split)
     prof_end(h, s);
     if (h->list) {
         prof_begin(h, SPH_KIND_LISTS, s);
-        CUDA_TRY(h, launch_scan((const unsigned*)h->nbr, h->n, h->noff_part, h->noff, s, &h->launches));
+        CUDA_TRY(h, launch_scan((unsigned*)h->nbr, h->n, h->noff_part, h->noff, false, s, &h->launches));
         CUDA_TRY(h, launch_fill_lists(h->pos_s, h->cell_start, h->sc, h->noff, h->list, h->list_cap, h->err, s,
                                       &h->launches));
         prof_end(h, s);

@@ -139,9 +139,10 @@ k_scan_reduce(const unsigned* __restrict__ in, int n, unsigned* __restrict__ par
     if (threadIdx.x == 0) part[blockIdx.x] = total;
 }
 
-// One block: exclusive scan of the tile totals in place; part[nparts] =
-// total.  1024 values per round: a shuffle scan in each warp, then of the
-// 32 warp totals by the first warp.
+// One block: exclusive scan of the tile totals in place (grids of so many
+// tiles that adding up those before it would hold every block).  1024 values
+// per round: a shuffle scan in each warp, then of the 32 warp totals by the
+// first warp.
 __global__ void __launch_bounds__(1024) k_scan_parts(unsigned* __restrict__ part, int nparts)
 {
     __shared__ unsigned sh_w[32];
@@ -175,7 +176,6 @@ __global__ void __launch_bounds__(1024) k_scan_parts(unsigned* __restrict__ part
         carry += carry_sh;
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[nparts] = carry;
 }
 
 // Element e of a tile lives at sh[e + e / 32]: one padding word per 32
@@ -184,9 +184,13 @@ __global__ void __launch_bounds__(1024) k_scan_parts(unsigned* __restrict__ part
 // conflicts (without it the second phase is a 16-way conflict).
 __device__ __forceinline__ int scan_pad(int e) { return e + (e >> 5); }
 
+// out[i] = the counts before i, out[n] = their total.  SUM: part holds the
+// tiles' totals and each block adds up those before its own (otherwise part
+// is already scanned).  zero: the counts are reset for the next histogram
+// (each is read by its own block alone).
+template <bool SUM>
 __global__ void __launch_bounds__(SCAN_THREADS)
-k_scan_tiles(const unsigned* __restrict__ in, int n, const unsigned* __restrict__ part,
-             unsigned* __restrict__ out)
+k_scan_tiles(unsigned* __restrict__ in, int n, const unsigned* __restrict__ part, unsigned* __restrict__ out, int zero)
 {
     __shared__ unsigned sh[SCAN_TILE + SCAN_TILE / 32];
     __shared__ unsigned sh_warp[SCAN_THREADS / 32];
@@ -196,7 +200,22 @@ k_scan_tiles(const unsigned* __restrict__ in, int n, const unsigned* __restrict_
         int idx = base + k * SCAN_THREADS + threadIdx.x;
         sh[scan_pad(k * SCAN_THREADS + threadIdx.x)] = idx < n ? in[idx] : 0u;
     }
+    unsigned before = 0;
+    if (SUM) {
+        for (int k = threadIdx.x; k < (int)blockIdx.x; k += SCAN_THREADS) before += __ldg(part + k);
+        unsigned dummy;
+        before = block_exclusive_scan(before, &dummy, sh_warp);
+    } else {
+        before = __ldg(part + blockIdx.x);
+    }
     __syncthreads();
+    if (zero) {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            int idx = base + k * SCAN_THREADS + threadIdx.x;
+            if (idx < n) in[idx] = 0u;
+        }
+    }
     unsigned local[SCAN_ITEMS];
     unsigned sum = 0;
 #pragma unroll
@@ -205,8 +224,8 @@ k_scan_tiles(const unsigned* __restrict__ in, int n, const unsigned* __restrict_
         sum += local[k];
     }
     unsigned prefix;
-    block_exclusive_scan(sum, &prefix, sh_warp);
-    prefix += part[blockIdx.x];
+    const unsigned total = block_exclusive_scan(sum, &prefix, sh_warp);
+    prefix += before;
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
         sh[scan_pad(threadIdx.x * SCAN_ITEMS + k)] = prefix;
@@ -218,23 +237,28 @@ k_scan_tiles(const unsigned* __restrict__ in, int n, const unsigned* __restrict_
         int idx = base + k * SCAN_THREADS + threadIdx.x;
         if (idx < n) out[idx] = sh[scan_pad(k * SCAN_THREADS + threadIdx.x)];
     }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + total;
 }
 
-__global__ void k_scan_total(const unsigned* __restrict__ part, int nparts, unsigned* __restrict__ out, int n)
-{
-    out[n] = part[nparts];
-}
+// Two launches up to this many tiles (33.5M cells; the large tank's grid has
+// 1,430): a block adds up to 32 totals per thread.  As three launches and a
+// fourth for the grand total the scan was a quarter of a small step's chain.
+constexpr int SCAN_SUM_MAX = 8192;
 
-cudaError_t launch_scan(const unsigned* counts, int n, unsigned* part, unsigned* start,
-                        cudaStream_t s, long long* launches)
+cudaError_t launch_scan(unsigned* counts, int n, unsigned* part, unsigned* start, bool zero, cudaStream_t s,
+                        long long* launches)
 {
     if (n <= 0) return cudaSuccess;
     int np = scan_parts(n);
     k_scan_reduce<<<np, SCAN_THREADS, 0, s>>>(counts, n, part);
-    k_scan_parts<<<1, 1024, 0, s>>>(part, np);
-    k_scan_tiles<<<np, SCAN_THREADS, 0, s>>>(counts, n, part, start);
-    k_scan_total<<<1, 1, 0, s>>>(part, np, start, n);
-    *launches += 4;
+    if (np <= SCAN_SUM_MAX) {
+        k_scan_tiles<true><<<np, SCAN_THREADS, 0, s>>>(counts, n, part, start, zero);
+        *launches += 2;
+    } else {
+        k_scan_parts<<<1, 1024, 0, s>>>(part, np);
+        k_scan_tiles<false><<<np, SCAN_THREADS, 0, s>>>(counts, n, part, start, zero);
+        *launches += 3;
+    }
     return cudaGetLastError();
 }
 
@@ -283,193 +307,20 @@ cudaError_t launch_scatter(const unsigned* key, const unsigned* rank, const unsi
 
 // ------------------------------------------------ per-cell sort + gather
 
-constexpr int SORT_WARPS = 8;
-constexpr int SORT_SMEM = 128;     // cells up to this size are ranked by one warp
-constexpr int BIG_THREADS = 1024;  // larger cells: one block, bitonic sort in smem
-constexpr int BIG_CAP = 16384;     // elements of a block sort (128 KiB of smem)
-// blocks of k_cellsort_big: one per multiprocessor (they loop over the queued cells)
-
-// One warp per cell.  tmp[start[c] ..) holds the storage indices of the
-// cell's particles in arbitrary order; each is ranked by particle id and its
-// pos/vel copied to start[c] + rank.  The attached particle of boid b
-// records its sorted slot in slot_of_boid[b].  Cells with more than
-// SORT_SMEM entries are queued in big_list for k_cellsort_big.
-__global__ void __launch_bounds__(SORT_WARPS * 32)
-k_cellsort_gather(const unsigned* __restrict__ start, int ncells, const int* __restrict__ tmp,
-                  const float4* __restrict__ pos_in, const float4* __restrict__ vel_in,
-                  float4* __restrict__ pos_out, float4* __restrict__ vel_out, int nb,
-                  int* __restrict__ slot_of_boid, int* __restrict__ big_list, unsigned* __restrict__ big_count)
-{
-    __shared__ int sh_id[SORT_WARPS][SORT_SMEM];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int c = blockIdx.x * SORT_WARPS + warp;
-    if (c >= ncells) return;
-    unsigned s0 = start[c];
-    int n = (int)(start[c + 1] - s0);
-    if (n == 0) return;
-    if (n <= 32) {
-        int src = 0, id = 0x7fffffff;
-        if (lane < n) {
-            src = tmp[s0 + lane];
-            id = id_of(pos_in[src]);
-        }
-        int r = 0;
-        for (int k = 0; k < n; ++k) {
-            int o = __shfl_sync(FULL, id, k);
-            r += o < id;
-        }
-        if (lane < n) {
-            unsigned dst = s0 + (unsigned)r;
-            pos_out[dst] = pos_in[src];
-            vel_out[dst] = vel_in[src];
-            if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
-        }
-        return;
-    }
-    if (n > SORT_SMEM) {
-        if (lane == 0) big_list[atomicAdd(big_count, 1u)] = c;
-        return;
-    }
-    for (int e = lane; e < n; e += 32) sh_id[warp][e] = id_of(pos_in[tmp[s0 + e]]);
-    __syncwarp();
-    for (int e = lane; e < n; e += 32) {
-        int src = tmp[s0 + e];
-        int id = sh_id[warp][e];
-        int r = 0;
-        for (int k = 0; k < n; ++k) r += sh_id[warp][k] < id;
-        unsigned dst = s0 + (unsigned)r;
-        pos_out[dst] = pos_in[src];
-        vel_out[dst] = vel_in[src];
-        if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
-    }
-}
-
-// One block per queued large cell: (id, storage index) pairs sorted by a
-// bitonic network in shared memory, then gathered.  Cells beyond BIG_CAP are
-// ranked by counting straight from global memory.
-__global__ void __launch_bounds__(BIG_THREADS)
-k_cellsort_big(const unsigned* __restrict__ start, const int* __restrict__ big_list,
-               const unsigned* __restrict__ big_count, const int* __restrict__ tmp,
-               const float4* __restrict__ pos_in, const float4* __restrict__ vel_in,
-               float4* __restrict__ pos_out, float4* __restrict__ vel_out, int nb,
-               int* __restrict__ slot_of_boid, const int* __restrict__ tmp_id, float* __restrict__ soa,
-               size_t soa_st)
-{
-    extern __shared__ unsigned long long sh_kv[];
-    // id of the entry at sorted-scratch position e (from tmp_id when given)
-    auto id_at = [&](unsigned e) { return tmp_id ? tmp_id[e] : id_of(pos_in[tmp[e]]); };
-    auto put = [&](unsigned dst, int src) {
-        const float4 p = pos_in[src];
-        pos_out[dst] = p;
-        vel_out[dst] = vel_in[src];
-        if (soa) {
-            soa[dst] = p.x;
-            soa[soa_st + dst] = p.y;
-            soa[2 * soa_st + dst] = p.z;
-        }
-    };
-    const unsigned nbig = *big_count;
-    for (unsigned b = blockIdx.x; b < nbig; b += gridDim.x) {
-        const int c = big_list[b];
-        const unsigned s0 = start[c];
-        const int n = (int)(start[c + 1] - s0);
-        if (n <= BIG_CAP) {
-            int P = 1;
-            while (P < n) P <<= 1;
-            for (int e = threadIdx.x; e < P; e += BIG_THREADS) {
-                unsigned long long v = ~0ull;
-                if (e < n) {
-                    int src = tmp[s0 + e];
-                    v = ((unsigned long long)(unsigned)id_at(s0 + e) << 32) | (unsigned)src;
-                }
-                sh_kv[e] = v;
-            }
-            __syncthreads();
-            for (int k = 2; k <= P; k <<= 1) {
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    for (int e = threadIdx.x; e < P; e += BIG_THREADS) {
-                        int partner = e ^ j;
-                        if (partner > e) {
-                            unsigned long long x = sh_kv[e], y = sh_kv[partner];
-                            bool ascending = (e & k) == 0;
-                            if ((x > y) == ascending) {
-                                sh_kv[e] = y;
-                                sh_kv[partner] = x;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
-            for (int e = threadIdx.x; e < n; e += BIG_THREADS) {
-                unsigned long long v = sh_kv[e];
-                int src = (int)(unsigned)(v & 0xffffffffull);
-                int id = (int)(unsigned)(v >> 32);
-                unsigned dst = s0 + (unsigned)e;
-                put(dst, src);
-                if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
-            }
-        } else {
-            for (int e = threadIdx.x; e < n; e += BIG_THREADS) {
-                int src = tmp[s0 + e];
-                int id = id_at(s0 + e);
-                int r = 0;
-                for (int k = 0; k < n; ++k) r += id_at(s0 + k) < id;
-                unsigned dst = s0 + (unsigned)r;
-                put(dst, src);
-                if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// One-time kernel attributes (the block sort's 128 KiB of shared memory);
-// called when a handle is created, before any stream capture.
-cudaError_t prepare_kernels()
-{
-    static bool done = false;
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_cellsort_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         BIG_CAP * (int)sizeof(unsigned long long));
-    if (e == cudaSuccess) done = true;
-    return e;
-}
-
-cudaError_t launch_cellsort_gather(const unsigned* start, int ncells, const int* tmp,
-                                   const float4* pos_in, const float4* vel_in, float4* pos_out,
-                                   float4* vel_out, int nb, int* slot_of_boid, int* big_list,
-                                   unsigned* big_count, cudaStream_t s, long long* launches)
-{
-    if (ncells <= 0) return cudaSuccess;
-    cudaError_t e = prepare_kernels();
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(big_count, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    int blocks = (ncells + SORT_WARPS - 1) / SORT_WARPS;
-    k_cellsort_gather<<<blocks, SORT_WARPS * 32, 0, s>>>(start, ncells, tmp, pos_in, vel_in, pos_out,
-                                                         vel_out, nb, slot_of_boid, big_list, big_count);
-    k_cellsort_big<<<sm_count(), BIG_THREADS, BIG_CAP * sizeof(unsigned long long), s>>>(
-        start, big_list, big_count, tmp, pos_in, vel_in, pos_out, vel_out, nb, slot_of_boid, nullptr, nullptr, 0);
-    *launches += 2;
-    return cudaGetLastError();
-}
-
 // One thread per sorted slot: the thread of slot s takes the storage index
-// tmp[s] of its cell, ranks its id tmp_id[s] against the cell's other ids
-// (a contiguous run of tmp_id) and moves pos/vel to start[c] + rank, also
-// writing x, y, z to the SoA copy (soa, soa_st floats per axis).  Cells with
-// more than SLOT_SMALL entries are queued (by the thread of their first
-// slot) for k_cellsort_big.  Suited to grids of small cells (a few particles
-// each).
-constexpr int SLOT_SMALL = 128;  // compressed fluid fills h/2 cells with 60-100 particles
-
+// tmp[s] of its cell, ranks its id tmp_id[s] against the cell's other ids (a
+// contiguous run of tmp_id, read by its threads together) and moves pos/vel
+// to start[c] + rank, also writing x, y, z to the SoA copy (soa, soa_st
+// floats per axis; may be NULL).  The attached particle of boid b records its
+// sorted slot in slot_of_boid[b].  A cell of n entries costs n reads per
+// entry, which holds for any n: the entries are spread over the chip (a cell
+// of 2,000 boids, the densest of the large tank's, takes 2,000 cached reads).
 __global__ void __launch_bounds__(256)
 k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict__ key, int n,
                  const int* __restrict__ tmp, const int* __restrict__ tmp_id, const float4* __restrict__ pos_in,
                  const float4* __restrict__ vel_in, float4* __restrict__ pos_out,
                  float4* __restrict__ vel_out, float* __restrict__ soa, size_t soa_st, int nb,
-                 int* __restrict__ slot_of_boid, int* __restrict__ big_list, unsigned* __restrict__ big_count)
+                 int* __restrict__ slot_of_boid)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
@@ -477,10 +328,6 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
     const unsigned c = key[src];
     const unsigned s0 = start[c];
     const int nc = (int)(start[c + 1] - s0);
-    if (nc > SLOT_SMALL) {
-        if ((unsigned)s == s0) big_list[atomicAdd(big_count, 1u)] = (int)c;
-        return;
-    }
     const int id = tmp_id[s];
     int r = 0;
     for (int k = 0; k < nc; ++k) r += __ldg(tmp_id + s0 + k) < id;
@@ -488,28 +335,23 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
     const float4 p = pos_in[src];
     pos_out[dst] = p;
     vel_out[dst] = vel_in[src];
-    soa[dst] = p.x;
-    soa[soa_st + dst] = p.y;
-    soa[2 * soa_st + dst] = p.z;
+    if (soa) {
+        soa[dst] = p.x;
+        soa[soa_st + dst] = p.y;
+        soa[2 * soa_st + dst] = p.z;
+    }
     if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
 }
 
-cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, int ncells,
-                                  const int* tmp, const int* tmp_id, const float4* pos_in, const float4* vel_in,
+cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, const int* tmp,
+                                  const int* tmp_id, const float4* pos_in, const float4* vel_in,
                                   float4* pos_out, float4* vel_out, float* soa, int nb, int* slot_of_boid,
-                                  int* big_list, unsigned* big_count, cudaStream_t s, long long* launches)
+                                  cudaStream_t s, long long* launches)
 {
-    if (n <= 0 || ncells <= 0) return cudaSuccess;
-    cudaError_t e = prepare_kernels();
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(big_count, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    const size_t st = soa_stride((size_t)n);
+    if (n <= 0) return cudaSuccess;
     k_cellsort_slots<<<(n + 255) / 256, 256, 0, s>>>(start, key, n, tmp, tmp_id, pos_in, vel_in, pos_out, vel_out,
-                                                     soa, st, nb, slot_of_boid, big_list, big_count);
-    k_cellsort_big<<<sm_count(), BIG_THREADS, BIG_CAP * sizeof(unsigned long long), s>>>(
-        start, big_list, big_count, tmp, pos_in, vel_in, pos_out, vel_out, nb, slot_of_boid, tmp_id, soa, st);
-    *launches += 2;
+                                                     soa, soa_stride((size_t)n), nb, slot_of_boid);
+    ++*launches;
     return cudaGetLastError();
 }
 

@@ -324,14 +324,11 @@ struct WarpRows {
 
 // ---------------------------------------------------------------- launchers
 
-// One-time kernel attributes; call before any stream capture.
-cudaError_t prepare_kernels();
-
-// Exclusive scan of n counts into start[0..n] (start[n] = total).  part must
-// hold scan_parts(n) + 1 entries.
+// Exclusive scan of n counts into start[0..n] (start[n] = total); with zero the
+// counts are reset.  part must hold scan_parts(n) entries.
 int scan_parts(int n);
-cudaError_t launch_scan(const unsigned* counts, int n, unsigned* part, unsigned* start,
-                        cudaStream_t s, long long* launches);
+cudaError_t launch_scan(unsigned* counts, int n, unsigned* part, unsigned* start, bool zero, cudaStream_t s,
+                        long long* launches);
 
 // The uniform grid over [mn, mx] with cells of size dx along x and d along
 // y and z (dim = ceil((mx - mn) / size) per axis, inv = fl(1 / size));
@@ -355,20 +352,14 @@ cudaError_t launch_scatter(const unsigned* key, const unsigned* rank, const unsi
 // The same, also tmp_id[dst] = id of the particle (pos.w).
 cudaError_t launch_scatter_ids(const unsigned* key, const unsigned* rank, const unsigned* start, const float4* pos,
                                int n, int* tmp, int* tmp_id, cudaStream_t s, long long* launches);
-// Per-cell sort by particle id + gather.  big_list (ncells ints) and
-// big_count (one u32) are scratch for the cells too large for one warp.
-cudaError_t launch_cellsort_gather(const unsigned* start, int ncells, const int* tmp,
-                                   const float4* pos_in, const float4* vel_in, float4* pos_out,
-                                   float4* vel_out, int nb, int* slot_of_boid, int* big_list,
-                                   unsigned* big_count, cudaStream_t s, long long* launches);
-// The same with one thread per sorted slot (for grids of small cells); key
-// holds the cell of every storage slot, n the number of particles.
-// tmp_id: the ids beside tmp (launch_scatter_ids); soa: the SoA copy of
+// Per-cell sort by particle id + gather, a thread per sorted slot; key holds
+// the cell of every storage slot, n the number of particles.  tmp_id: the
+// ids beside tmp (launch_scatter_ids); soa (may be NULL): the SoA copy of
 // pos_out (soa_stride(n) floats per axis), written as well.
-cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, int ncells,
-                                  const int* tmp, const int* tmp_id, const float4* pos_in, const float4* vel_in,
+cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, const int* tmp,
+                                  const int* tmp_id, const float4* pos_in, const float4* vel_in,
                                   float4* pos_out, float4* vel_out, float* soa, int nb, int* slot_of_boid,
-                                  int* big_list, unsigned* big_count, cudaStream_t s, long long* launches);
+                                  cudaStream_t s, long long* launches);
 cudaError_t launch_slot_keys(const unsigned* start, int ncells, unsigned* slot_key, cudaStream_t s,
                              long long* launches);
 

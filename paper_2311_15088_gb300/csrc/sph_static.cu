@@ -206,7 +206,7 @@ int sph_bin_static(const sph_params* p, int n, const float* pos4, unsigned* keys
     if (e == cudaSuccess) e = cudaMemsetAsync(big_count, 0, 8, s);
     if (e == cudaSuccess) e = launch_keys(reinterpret_cast<const float4*>(pos4), n, g, p->box_min, p->box_max,
                                           keys_out, rank, count, err, s, &launches);
-    if (e == cudaSuccess) e = launch_scan(count, g.ncells, part, cell_start_out, s, &launches);
+    if (e == cudaSuccess) e = launch_scan(count, g.ncells, part, cell_start_out, false, s, &launches);
     if (e == cudaSuccess) e = launch_scatter(keys_out, rank, cell_start_out, n, perm_out, s, &launches);
     if (e == cudaSuccess) {
         k_sort_cells_index<<<(g.ncells + SORT_WARPS - 1) / SORT_WARPS, SORT_WARPS * 32, 0, s>>>(

@@ -404,6 +404,21 @@ cudaError_t launch_density(const float4* pos, const float4* vel, const SoaPos& x
                            const Scenes& sc, const Tuning& t, float* rho, float2* ab, float4* prec, int* nbr,
                            uint2* seg, int* nseg, int* ncand, const int* list, const unsigned* list_len,
                            unsigned* err, cudaStream_t s, long long* launches);
+// The boid rules' arguments: the sorted boids and their cells, the obstacle
+// grid, F_b (by boid), the particles' sorted velocities of the step (the
+// attached particles' own, read by the literal coupling), and what the rules
+// write: the boids, and their attached particles' next state and keys.
+struct BoidArgs {
+    const float4 *bpos_s, *bvel_s;
+    const unsigned* bstart;
+    const float4* obst;
+    const float4* fb;
+    const float4* vel_s;
+    float4 *bpos, *bvel, *pos_next, *vel_next;
+    const int* slot_of_boid;
+    unsigned *key, *rank, *count, *err;
+};
+
 // The step's force pass: F_b of every boid (bmask NULL) or of the boids with
 // bmask[b] != 0 (their fb.w = 1), a warp per boid, also stored to acc at the
 // attached slot when acc is given; with fluid = true also every fluid
@@ -420,8 +435,8 @@ cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* ve
                           const Tuning& t, const unsigned* list, const unsigned* list_off, size_t list_cap,
                           bool boids, bool fluid, const int* slot_of_boid, const int* bmask, float4* fb,
                           float4* acc, int* touched, float4* infl, float4* pos_next, float4* vel_next,
-                          unsigned* key, unsigned* rank, unsigned* count, unsigned* err, cudaStream_t s,
-                          long long* launches);
+                          unsigned* key, unsigned* rank, unsigned* count, unsigned* err, const BoidArgs* rules,
+                          cudaStream_t s, long long* launches);
 // Both neighbour passes in one cooperative launch (t.pipe_tile > 0):
 // density over tiles of sorted slots, a bounded grid barrier
 // (SPH_DEV_TIMEOUT if it gives up), then F_b of the boids and the force
@@ -455,14 +470,13 @@ cudaError_t launch_boid_keys(const float4* bpos, const Scenes& sc, unsigned* bke
 // then n_box x (min, max) floats, device memory.
 cudaError_t launch_obstacle_grid(const StepConst& c, const float* shapes, int n_sphere, int n_box, float half_diag,
                                  float4* grid, cudaStream_t s, long long* launches);
-// vel_s: the particles' sorted velocities of the step (the attached
-// particles' own velocities, read by the literal coupling).
-cudaError_t launch_boid_rules(const float4* bpos_s, const float4* bvel_s, const unsigned* bstart,
-                              const float4* obst, const Scenes& sc, const float4* fb, const float4* vel_s,
-                              float4* bpos, float4* bvel,
-                              float4* pos_next, float4* vel_next, const int* slot_of_boid,
-                              unsigned* key, unsigned* rank, unsigned* count, unsigned* err,
-                              cudaStream_t s, long long* launches);
+cudaError_t launch_boid_rules(const BoidArgs& a, const Scenes& sc, cudaStream_t s, long long* launches);
+// The boids' binning in one launch, where they are few (at most 1,024 in
+// fewer than 8,192 cells): bstart (nbcells + 1 starts) and the sorted copies.
+bool boid_bin_is_small(const Scenes& sc, int nbcells);
+cudaError_t launch_boid_bin_small(const float4* bpos, const float4* bvel, const Scenes& sc, int nbcells,
+                                  float4* bpos_s, float4* bvel_s, unsigned* bstart, cudaStream_t s,
+                                  long long* launches);
 
 // Surrogate inputs and outputs (sph_features.cu).  The feature grid pass
 // (every fluid particle into the integer sums of its feature cell; grid:

@@ -16,7 +16,7 @@
 // z, y order, x ascending, each row clipped to the sphere), so its float32
 // sums have a fixed order that depends only on the state.  Neighbouring
 // threads share cells, so the candidate loads are served by L1.
-#include "sph_internal.cuh"
+#include "sph_boids.cuh"
 
 namespace sphk {
 
@@ -429,8 +429,9 @@ __device__ __forceinline__ float2 dxy_of(const float4& pj, float2 nxy)
 // candidates by flat index (lane l: candidates l, l + 32, ... in walk
 // order), each keeping its own sum, and a butterfly adds the 32 sums (a
 // fixed order).
+// Returns F_b on lane 0.
 template <bool COH>
-__device__ __forceinline__ void boid_fb_warp(int b, int lane, const float4* __restrict__ pos,
+__device__ __forceinline__ float4 boid_fb_warp(int b, int lane, const float4* __restrict__ pos,
                                              const float4* __restrict__ vel, const float* __restrict__ rho,
                                              const float2* __restrict__ ab, const unsigned* __restrict__ start,
                                              const Scenes& sc, const int* __restrict__ slot_of_boid,
@@ -474,12 +475,14 @@ __device__ __forceinline__ void boid_fb_warp(int b, int lane, const float4* __re
         ay += __shfl_xor_sync(FULL, ay, o);
         az += __shfl_xor_sync(FULL, az, o);
     }
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
     if (lane == 0) {
         const float inv_rho = 1.0f / ldd<COH>(rho + i);
-        const float4 f = make_float4(ax * inv_rho, ay * inv_rho, az * inv_rho, 0.0f);
+        f = make_float4(ax * inv_rho, ay * inv_rho, az * inv_rho, 0.0f);
         fb[b] = make_float4(f.x, f.y, f.z, bmask ? 1.0f : 0.0f);
         if (acc) acc[i] = f;
     }
+    return f;
 }
 
 // The arguments of the force pass (k_forces and the fused pipeline).
@@ -708,14 +711,24 @@ __device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
 
 // The step's force pass.  The first boid_blocks blocks compute F_b, a warp
 // per boid (boid_fb_warp; F_b also goes to acc at the attached slot when
-// acc is given); they come first in the grid so that these latency-bound
-// warps run alongside the fluid blocks.  The remaining blocks (possibly
+// acc is given) and, with the rules' arguments, then run the boid's rules;
+// they come first in the grid so that these latency-bound warps run
+// alongside the fluid blocks.  The remaining blocks (possibly
 // none) take a particle per thread (force_particle).
 __global__ void __launch_bounds__(512)
-k_forces(ForceArgs a, int boid_blocks)
+k_forces(ForceArgs a, int boid_blocks, BoidArgs r)
 {
     if ((int)blockIdx.x < boid_blocks) {
-        const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        if (r.bpos_s) {  // with the rules: the boid at sorted boid slot b
+            if (b >= a.sc.nb_all) return;  // whole warps
+            const int s = b, lane = threadIdx.x & 31;
+            b = id_of(r.bpos_s[s]);
+            const float4 f = boid_fb_warp<false>(b, lane, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
+                                                 nullptr, a.fb, a.acc);
+            boid_rules_warp(r, a.sc, s, lane, [&](int) { return f; });
+            return;
+        }
         if (b < a.sc.nb_all && !(a.bmask && !a.bmask[b]))  // uniform per warp
             boid_fb_warp<false>(b, threadIdx.x & 31, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
                                 a.bmask, a.fb, a.acc);
@@ -735,8 +748,8 @@ cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* ve
                           const Tuning& t, const unsigned* list, const unsigned* list_off, size_t list_cap,
                           bool boids, bool fluid, const int* slot_of_boid, const int* bmask, float4* fb,
                           float4* acc, int* touched, float4* infl, float4* pos_next, float4* vel_next,
-                          unsigned* key, unsigned* rank, unsigned* count, unsigned* err, cudaStream_t s,
-                          long long* launches)
+                          unsigned* key, unsigned* rank, unsigned* count, unsigned* err, const BoidArgs* rules,
+                          cudaStream_t s, long long* launches)
 {
     const unsigned cap = list_cap > 0xffffffffu ? 0xffffffffu : (unsigned)list_cap;
     const int warps = t.block / 32;
@@ -746,7 +759,9 @@ cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* ve
     if (boid_blocks + fluid_blocks == 0) return cudaSuccess;
     const ForceArgs a{pos, xyz, vel, rho, ab, prec, start, t.use_seg ? seg : nullptr, nseg, sc, list, list_off, cap,
                       slot_of_boid, bmask, fb, acc, touched, infl, pos_next, vel_next, key, rank, count, err};
-    k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks);
+    BoidArgs r{};
+    if (rules) r = *rules;
+    k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks, r);
     ++*launches;
     return cudaGetLastError();
 }

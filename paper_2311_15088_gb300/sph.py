@@ -149,6 +149,13 @@ def make_params(p: dict) -> SphParams:
     return s
 
 
+def _stream_of(torch, device) -> int:
+    """The cudaStream_t of torch's current stream on device (the number alone:
+    making torch's Stream object costs some 3 us, more than a launch)."""
+    index = device.index if device.index is not None else torch._C._cuda_getDevice()
+    return torch._C._cuda_getCurrentRawStream(index)
+
+
 # ----------------------------------------------------------- C-ABI names
 
 def sph_workspace_size(params: dict, n_fluid: int, n_boid: int) -> int:
@@ -503,7 +510,7 @@ class Mlp:
 
     @property
     def stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
+        return _stream_of(self.torch, self.device)
 
     def _pad(self, x, width, dtype):
         t = self.torch
@@ -624,7 +631,7 @@ class Scene:
 
     @property
     def stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
+        return _stream_of(self.torch, self.device)
 
     def _dev4(self, a, n):
         t = self.torch.as_tensor(np.asarray(a, np.float32) if not self.torch.is_tensor(a) else a)

@@ -1490,7 +1490,7 @@ int sph_voxel_density(sph_handle* h, const float* origin, const int* dims, float
 
 struct McLayout {
     long long ncubes;
-    size_t tile_off, tile_count, count, cases, total;
+    size_t tile_off, tile_count, cases, total;
 };
 
 static int mc_layout(const int* dims, McLayout* L)
@@ -1503,8 +1503,7 @@ static int mc_layout(const int* dims, McLayout* L)
     const size_t nt = (size_t)(n > 0 ? mc_tiles(n) : 1);
     L->tile_off = 0;
     L->tile_count = up(nt * sizeof(unsigned long long));
-    L->count = L->tile_count + up(nt * sizeof(unsigned));
-    L->cases = L->count + 256;
+    L->cases = L->tile_count + up(nt * sizeof(unsigned));
     L->total = L->cases + up((size_t)(n > 0 ? n : 1));
     return SPH_OK;
 }
@@ -1538,12 +1537,10 @@ int sph_marching_cubes(const float* phi, const int* dims, const float* origin, f
     if (e != cudaSuccess) return fail(nullptr, SPH_ERR_CUDA, "marching-cubes tables: %s", cudaGetErrorString(e));
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t* w = (uint8_t*)workspace;
-    unsigned* count = (unsigned*)(w + L.count);
     long long launches = 0;
     e = launch_marching_cubes(phi, dims, origin, spacing, iso, (unsigned char*)(w + L.cases), (unsigned*)(w + L.tile_count),
-                              (unsigned long long*)(w + L.tile_off), count, tris, (unsigned long long)max_tris, s,
+                              (unsigned long long*)(w + L.tile_off), ntri, tris, (unsigned long long)max_tris, s,
                               &launches);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ntri, count, sizeof(unsigned), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return fail(nullptr, SPH_ERR_CUDA, "marching cubes: %s", cudaGetErrorString(e));
     return SPH_OK;
 }

@@ -197,9 +197,10 @@ k_density(const float4* __restrict__ pos, const float4* __restrict__ vel, SoaPos
 // list[0 .. *list_len), built on the device).  The lanes fetch the walk's rows
 // together, cut them into pieces of at most 32 slots (a segment each) and
 // test the pieces' candidates side by side by flat index; the hits are added
-// in walk order by the same fused multiply-adds as the one-thread pass (the
-// lanes pass the terms by shuffles), and the lane of a piece gathers its
-// mask from the rounds' ballots.  Same bits as density_at.  Bound by latency:
+// in walk order by the same fused multiply-adds as the one-thread pass (every
+// lane reads the terms, packed, from shared memory: passed one by one by
+// shuffles they were most of the instructions), and the lane of a piece
+// gathers its mask from the rounds' ballots.  Same bits as density_at.  Bound by latency:
 // 4,112 particles take 12 us where the one-thread pass takes 42 (16 blocks,
 // each thread some 100 candidates in series).
 template <bool SEG, bool LIST>
@@ -209,7 +210,12 @@ k_density_warp(const float4* __restrict__ pos, const float4* __restrict__ vel, c
                int* __restrict__ nbr, uint2* __restrict__ seg, int* __restrict__ nseg, int* __restrict__ ncand,
                const int* __restrict__ list, const unsigned* __restrict__ list_len, unsigned* __restrict__ err)
 {
+    // a round's terms h2 - r2, the hits' first and in order, zeros behind them
+    // (two rounds' worth: one is read while the next is written)
+    __shared__ __align__(16) float s_term[4][2][32];
     const int lane = threadIdx.x & 31;
+    float(*const term)[32] = s_term[threadIdx.x >> 5];
+    int round = 0;
     const int nw = gridDim.x * (blockDim.x >> 5);
     const int len = LIST ? (int)min(*list_len, (unsigned)sc.n_all) : sc.n_all;
     for (int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < len; w += nw) {
@@ -274,12 +280,20 @@ k_density_warp(const float4* __restrict__ pos, const float4* __restrict__ vel, c
                         const unsigned plen = rows.s1 - rows.s0;
                         mine |= in & (plen < 32u ? (1u << plen) - 1u : FULL);
                     }
-                    const float tt = __fmul_rn(t, t);
-                    while (m) {  // the hits in walk order, one fused multiply-add each
-                        const int q = __ffs((int)m) - 1;
-                        m &= m - 1u;
-                        sum = fmaf(__shfl_sync(FULL, tt, q), __shfl_sync(FULL, t, q), sum);
+                    // the hits in walk order, one fused multiply-add each; a
+                    // zero adds +0 and changes no bit
+                    const int n = __popc(m), below = __popc(m & ((1u << lane) - 1u));
+                    float* const buf = term[round];
+                    buf[hit ? below : n + lane - below] = hit ? t : 0.0f;
+                    __syncwarp();
+                    for (int q = 0; q < n; q += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(buf + q);
+                        sum = fmaf(__fmul_rn(v.x, v.x), v.x, sum);
+                        sum = fmaf(__fmul_rn(v.y, v.y), v.y, sum);
+                        sum = fmaf(__fmul_rn(v.z, v.z), v.z, sum);
+                        sum = fmaf(__fmul_rn(v.w, v.w), v.w, sum);
                     }
+                    round ^= 1;
                 }
                 if (SEG && !att_i) {
                     const unsigned has = __ballot_sync(FULL, mine != 0u);

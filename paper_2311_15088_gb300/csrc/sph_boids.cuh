@@ -59,19 +59,25 @@ __device__ __forceinline__ void boid_rules_warp(const BoidArgs& a, const Scenes&
             ++nv;
         }
     };
-    RowWalk walk(c.gb, c.wb, a.bstart + c.cb_base, pb.x, pb.y, pb.z);
-    unsigned s0, s1;
-    while (walk.next(s0, s1)) {
-        // lane l takes slots s0 + l, s0 + l + 32, ... in that order, two
-        // at a time so that both candidates' loads are in flight together
-        unsigned j = s0 + lane;
-        for (; j + 32 < s1; j += 64) {
-            const float4 pa = bpos_s[j], va = bvel_s[j];
-            const float4 pc = bpos_s[j + 32], vc = bvel_s[j + 32];
-            if (j != (unsigned)s) take(pa, va);
-            if (j + 32 != (unsigned)s) take(pc, vc);
+    // the lanes fetch the walk's rows together (a row after another, their
+    // start loads were most of a small school's time), then take each in turn
+    WarpRows rows(c.gb, c.wb, a.bstart + c.cb_base, pb.x, pb.y, pb.z);
+    for (int bt = 0; 32 * bt < rows.nrows; ++bt) {
+        const int n = rows.batch(bt);
+        for (int k = 0; k < n; ++k) {
+            unsigned s0, s1;
+            rows.row(k, s0, s1);
+            // lane l takes slots s0 + l, s0 + l + 32, ... in that order, two
+            // at a time so that both candidates' loads are in flight together
+            unsigned j = s0 + lane;
+            for (; j + 32 < s1; j += 64) {
+                const float4 pa = bpos_s[j], va = bvel_s[j];
+                const float4 pc = bpos_s[j + 32], vc = bvel_s[j + 32];
+                if (j != (unsigned)s) take(pa, va);
+                if (j + 32 != (unsigned)s) take(pc, vc);
+            }
+            if (j < s1 && j != (unsigned)s) take(bpos_s[j], bvel_s[j]);
         }
-        if (j < s1 && j != (unsigned)s) take(bpos_s[j], bvel_s[j]);
     }
     // obstacle avoidance: the obstacle-grid cells whose centre lies within
     // the visual range (the float32 predicate of the boid pairs), their mean

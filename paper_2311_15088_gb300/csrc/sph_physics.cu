@@ -528,32 +528,229 @@ struct ForceArgs {
     unsigned* __restrict__ err;
 };
 
-// The force pass of sorted slot i (i >= n_all: an idle lane): pair forces
-// with touched_by_boid and boid_influence, gravity, Euler-Cromer
-// integration, damped walls and the next step's cell keys.  A fluid
-// particle takes its pairs from (in this order of preference) the
-// neighbour list, the density pass's hit segments, or a walk that tests the
-// candidates again; all three visit the same pairs in the same order.
-// acc, touched and infl (the diagnostic fields) are written only when given
-// (all three or none); attached particles then record touched = 0 and
-// influence = 0 (attached pairs are excluded).  Every lane of the warp
-// must call it (warp-aggregated counting).
+// A particle's pair sums over its neighbours: the force, and the part and
+// number of attached ones.
+struct PairSums {
+    float2 axy = make_float2(0.f, 0.f), bxy = make_float2(0.f, 0.f);
+    float az = 0.f, bz = 0.f;
+    int touch = 0;
+};
+
+// The pair sums of fluid particle i (at pi) by one thread.  It takes its
+// pairs from (in this order of preference) the neighbour list, the density
+// pass's hit segments, or a walk that tests the candidates again; all three
+// visit the same pairs in the same order.
 template <bool COH>
-__device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
+__device__ __forceinline__ PairSums pair_sums(const ForceArgs& a, int i, const StepConst& c, const float4& pi)
 {
     const float4* __restrict__ pos = a.pos;
     const SoaPos& xyz = a.xyz;
     const float4* __restrict__ vel = a.vel;
-    const float* rho = a.rho;
     const float2* ab = a.ab;
     const float4* prec = a.prec;
-    const unsigned* __restrict__ start = a.start;
     const uint2* seg = a.seg;
     const int* nseg = a.nseg;
     const Scenes& sc = a.sc;
     const unsigned* __restrict__ list = a.list;
     const unsigned* __restrict__ list_off = a.list_off;
     const unsigned list_cap = a.list_cap;
+    unsigned* __restrict__ err = a.err;
+    const unsigned* cstart = a.start + c.c_base;
+    float2 axy = make_float2(0.f, 0.f), bxy = make_float2(0.f, 0.f);
+    float az = 0.f, bz = 0.f;
+    int touch = 0;
+    PairTerms T;
+    T.set(c, pi, __ldg(vel + i), ldd<COH>(ab + i).y);
+    const float2 nxy = make_float2(-pi.x, -pi.y);
+    // one neighbour j (r2 < h2) from its record (one 32-byte load); the
+    // particle itself and coincident particles (r2 = 0) add nothing
+    auto pair = [&](unsigned j) {
+        if (!SPH_IN_BOUNDS(j, sc.n_all, err)) return;  // a hit segment's slot
+        float4 q0, q1;
+        ld_rec<COH>(prec + 2 * (size_t)j, q0, q1);
+        const float2 dxy = dxy_of(q0, nxy);
+        const float dz = __fsub_rn(q0.z, pi.z);
+        const float r2 = pair_r2(dxy.x, dxy.y, dz);
+        float2 fxy;
+        float fz;
+        T.add(dxy, dz, r2, q1, make_float2(fabsf(q1.w), q0.w), fxy, fz);
+        if (r2 != 0.0f) {
+            axy = __fadd2_rn(axy, fxy);
+            az = __fadd_rn(az, fz);
+            if (__float_as_int(q1.w) < 0) {  // j is attached to a boid
+                ++touch;
+                bxy = __fadd2_rn(bxy, fxy);
+                bz = __fadd_rn(bz, fz);
+            }
+        }
+    };
+    unsigned o0 = 0, o1 = 0;
+    if (list) {
+        o0 = __ldg(list_off + i);
+        o1 = __ldg(list_off + i + 1);
+    }
+    const int ns = seg ? ldd<COH>(nseg + i) : SEG_CAP + 1;
+    if (list && o1 <= list_cap) {
+        // the neighbour list, in walk order (coincident particles skipped)
+        for (unsigned k = o0; k < o1; ++k) {
+            const unsigned j = __ldg(list + k);
+            const float4 pj = __ldg(pos + j);
+            if (pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z)) != 0.0f) pair(j);
+        }
+    } else if (ns <= SEG_CAP) {
+        // the density pass's hit segments: one pair per iteration, the
+        // next segment fetched while the current pair is evaluated
+        const uint2* __restrict__ mine = seg + (size_t)i * SEG_CAP;
+        uint2 cur = ns > 0 ? ldd<COH>(mine) : make_uint2(0u, 0u);
+        int k = 1;
+        while (cur.y) {
+            const unsigned j = cur.x + (unsigned)(__ffs(cur.y) - 1);
+            cur.y &= cur.y - 1u;
+            if (!cur.y && k < ns) cur = ldd<COH>(mine + k++);
+            pair(j);
+        }
+    } else {
+        // test a chunk of up to 32 candidates into a bit mask, then run
+        // the pair code over the set bits (slot pairs from the SoA copy,
+        // as in the density pass)
+        const float h2 = c.h2;
+        const float2 nx2 = make_float2(-pi.x, -pi.x), ny2 = make_float2(-pi.y, -pi.y),
+                     nz2 = make_float2(-pi.z, -pi.z);
+        const float2* __restrict__ X2 = reinterpret_cast<const float2*>(xyz.x);
+        const float2* __restrict__ Y2 = reinterpret_cast<const float2*>(xyz.y);
+        const float2* __restrict__ Z2 = reinterpret_cast<const float2*>(xyz.z);
+        auto test1 = [&](unsigned j) {
+            const float4 pj = __ldg(pos + j);
+            const float r2 = pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z));
+            return (unsigned)(r2 < h2 && r2 != 0.0f);
+        };
+        auto test2 = [&](float2 X, float2 Y, float2 Z) {
+            const float2 dx = __fadd2_rn(X, nx2), dy = __fadd2_rn(Y, ny2), dz = __fadd2_rn(Z, nz2);
+            const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+            return (unsigned)(r2.x < h2 && r2.x != 0.0f) | (unsigned)(r2.y < h2 && r2.y != 0.0f) << 1;
+        };
+        RowWalk walk(c.g, c.wg, cstart, pi.x, pi.y, pi.z);
+        unsigned s0, s1;
+        while (walk.next(s0, s1)) {
+            for (unsigned base = s0; base < s1; base += 32) {
+                const unsigned e = min(base + 32u, s1);
+                unsigned m = 0, j = base;
+                if (j & 1u) m = test1(j++);
+                const unsigned e2 = e & ~1u;
+                for (; j + 4 <= e2; j += 4) {
+                    const unsigned k = j >> 1;
+                    const float2 xa = __ldg(X2 + k), ya = __ldg(Y2 + k), za = __ldg(Z2 + k);
+                    const float2 xb = __ldg(X2 + k + 1), yb = __ldg(Y2 + k + 1), zb = __ldg(Z2 + k + 1);
+                    m |= test2(xa, ya, za) << (j - base);
+                    m |= test2(xb, yb, zb) << (j + 2 - base);
+                }
+                if (j < e2) {
+                    const unsigned k = j >> 1;
+                    m |= test2(__ldg(X2 + k), __ldg(Y2 + k), __ldg(Z2 + k)) << (j - base);
+                    j += 2;
+                }
+                if (j < e) m |= test1(j) << (j - base);
+                while (m) {
+                    const int t = __ffs(m) - 1;
+                    m &= m - 1u;
+                    pair(base + (unsigned)t);
+                }
+            }
+        }
+    }
+    PairSums s;
+    s.axy = axy;
+    s.bxy = bxy;
+    s.az = az;
+    s.bz = bz;
+    s.touch = touch;
+    return s;
+}
+
+// The same by a warp, from the hit segments: the lanes take the hits by
+// number (32 segments at a time), evaluate their pairs side by side and pass
+// them through shared memory (out: the warp's 32 entries), where every lane
+// adds them in walk order; same bits.  A list that did not fit is walked by
+// one lane (lane 0 then holds the result).
+__device__ __forceinline__ PairSums pair_sums_warp(const ForceArgs& a, int i, const StepConst& c, const float4& pi,
+                                                   float4* out)
+{
+    const int lane = threadIdx.x & 31;
+    const int ns = __ldg(a.nseg + i);
+    PairSums s;
+    if (ns > SEG_CAP) {
+        if (lane == 0) s = pair_sums<false>(a, i, c, pi);
+        return s;
+    }
+    PairTerms T;
+    T.set(c, pi, __ldg(a.vel + i), __ldg(a.ab + i).y);
+    const float2 nxy = make_float2(-pi.x, -pi.y);
+    const uint2* __restrict__ mine = a.seg + (size_t)i * SEG_CAP;
+    for (int k0 = 0; k0 < ns; k0 += 32) {
+        const uint2 g = k0 + lane < ns ? __ldg(mine + k0 + lane) : make_uint2(0u, 0u);
+        const int hits = __popc(g.y);
+        int inc = hits;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += u;
+        }
+        const int pre = inc - hits, total = __shfl_sync(FULL, inc, 31);
+        for (int h0 = 0; h0 < total; h0 += 32) {
+            const int h = min(h0 + lane, total - 1);
+            int lo = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {  // the last segment whose first hit is <= h
+                const int p = __shfl_sync(FULL, pre, lo + step);
+                if (p <= h) lo += step;
+            }
+            unsigned m = __shfl_sync(FULL, g.y, lo);
+            const unsigned first = __shfl_sync(FULL, g.x, lo);
+            for (int q = h - __shfl_sync(FULL, pre, lo); q > 0; --q) m &= m - 1u;  // to its q-th hit
+            const unsigned j = first + (unsigned)(__ffs((int)m) - 1);
+            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);  // w: the hit is of an attached particle
+            if (h0 + lane < total && SPH_IN_BOUNDS(j, a.sc.n_all, a.err)) {
+                float4 q0, q1;
+                ld_rec<false>(a.prec + 2 * (size_t)j, q0, q1);
+                const float2 dxy = dxy_of(q0, nxy);
+                const float dz = __fsub_rn(q0.z, pi.z);
+                const float r2 = pair_r2(dxy.x, dxy.y, dz);
+                float2 fxy;
+                float fz;
+                T.add(dxy, dz, r2, q1, make_float2(fabsf(q1.w), q0.w), fxy, fz);
+                // the particle itself and coincident ones add +0, which changes no bit
+                if (r2 != 0.0f) r = make_float4(fxy.x, fxy.y, fz, __float_as_int(q1.w) < 0 ? 1.0f : 0.0f);
+            }
+            __syncwarp();  // the round before is read
+            out[lane] = r;
+            __syncwarp();
+            const int n = min(32, total - h0);
+            for (int k = 0; k < n; ++k) {
+                const float4 v = out[k];
+                s.axy = __fadd2_rn(s.axy, make_float2(v.x, v.y));
+                s.az = __fadd_rn(s.az, v.z);
+                if (v.w != 0.0f) {  // uniform
+                    ++s.touch;
+                    s.bxy = __fadd2_rn(s.bxy, make_float2(v.x, v.y));
+                    s.bz = __fadd_rn(s.bz, v.z);
+                }
+            }
+        }
+    }
+    return s;
+}
+
+// The rest of the force pass of sorted slot i (i >= n_all: an idle lane)
+// from its pair sums: gravity, Euler-Cromer integration, damped walls and the
+// next step's cell keys.  acc, touched and infl (the diagnostic fields) are
+// written only when given (all three or none); attached particles then
+// record touched = 0 and influence = 0 (attached pairs are excluded).  Every
+// lane of the warp must call it (warp-aggregated counting).
+template <bool COH>
+__device__ __forceinline__ void integrate(const ForceArgs& a, int i, const PairSums& s)
+{
+    const Scenes& sc = a.sc;
+    const float4* __restrict__ vel = a.vel;
     float4* __restrict__ acc = a.acc;
     int* __restrict__ touched = a.touched;
     float4* __restrict__ infl = a.infl;
@@ -566,118 +763,14 @@ __device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
     const bool active = i < sc.n_all;
     const int ii = active ? i : 0;
     const StepConst& c = sc.c[scene_of(sc.pbase, sc.S, (unsigned)ii)];
-    const int nb_all = sc.nb_all;
-    const float4 pi = pos[ii];
-    const bool fluid = active && id_of(pi) >= nb_all;
-    const unsigned* cstart = start + c.c_base;
-
-    float2 axy = make_float2(0.f, 0.f), bxy = make_float2(0.f, 0.f);
-    float az = 0.f, bz = 0.f;
-    int touch = 0;
-    float rho_i = 1.0f;
+    const float4 pi = a.pos[ii];
+    const bool fluid = active && id_of(pi) >= sc.nb_all;
+    const float2 axy = s.axy, bxy = s.bxy;
+    float az = s.az;
+    const float bz = s.bz;
+    const int touch = s.touch;
+    const float rho_i = fluid ? ldd<COH>(a.rho + i) : 1.0f;
     bool clamped = false;
-    if (fluid) {
-        PairTerms T;
-        T.set(c, pi, __ldg(vel + i), ldd<COH>(ab + i).y);
-        rho_i = ldd<COH>(rho + i);
-        const float2 nxy = make_float2(-pi.x, -pi.y);
-        // one neighbour j (r2 < h2) from its record (one 32-byte load); the
-        // particle itself and coincident particles (r2 = 0) add nothing
-        auto pair = [&](unsigned j) {
-            if (!SPH_IN_BOUNDS(j, sc.n_all, err)) return;  // a hit segment's slot
-            float4 q0, q1;
-            ld_rec<COH>(prec + 2 * (size_t)j, q0, q1);
-            const float2 dxy = dxy_of(q0, nxy);
-            const float dz = __fsub_rn(q0.z, pi.z);
-            const float r2 = pair_r2(dxy.x, dxy.y, dz);
-            float2 fxy;
-            float fz;
-            T.add(dxy, dz, r2, q1, make_float2(fabsf(q1.w), q0.w), fxy, fz);
-            if (r2 != 0.0f) {
-                axy = __fadd2_rn(axy, fxy);
-                az = __fadd_rn(az, fz);
-                if (__float_as_int(q1.w) < 0) {  // j is attached to a boid
-                    ++touch;
-                    bxy = __fadd2_rn(bxy, fxy);
-                    bz = __fadd_rn(bz, fz);
-                }
-            }
-        };
-        unsigned o0 = 0, o1 = 0;
-        if (list) {
-            o0 = __ldg(list_off + i);
-            o1 = __ldg(list_off + i + 1);
-        }
-        const int ns = seg ? ldd<COH>(nseg + i) : SEG_CAP + 1;
-        if (list && o1 <= list_cap) {
-            // the neighbour list, in walk order (coincident particles skipped)
-            for (unsigned k = o0; k < o1; ++k) {
-                const unsigned j = __ldg(list + k);
-                const float4 pj = __ldg(pos + j);
-                if (pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z)) != 0.0f) pair(j);
-            }
-        } else if (ns <= SEG_CAP) {
-            // the density pass's hit segments: one pair per iteration, the
-            // next segment fetched while the current pair is evaluated
-            const uint2* __restrict__ mine = seg + (size_t)i * SEG_CAP;
-            uint2 cur = ns > 0 ? ldd<COH>(mine) : make_uint2(0u, 0u);
-            int k = 1;
-            while (cur.y) {
-                const unsigned j = cur.x + (unsigned)(__ffs(cur.y) - 1);
-                cur.y &= cur.y - 1u;
-                if (!cur.y && k < ns) cur = ldd<COH>(mine + k++);
-                pair(j);
-            }
-        } else {
-            // test a chunk of up to 32 candidates into a bit mask, then run
-            // the pair code over the set bits (slot pairs from the SoA copy,
-            // as in the density pass)
-            const float h2 = c.h2;
-            const float2 nx2 = make_float2(-pi.x, -pi.x), ny2 = make_float2(-pi.y, -pi.y),
-                         nz2 = make_float2(-pi.z, -pi.z);
-            const float2* __restrict__ X2 = reinterpret_cast<const float2*>(xyz.x);
-            const float2* __restrict__ Y2 = reinterpret_cast<const float2*>(xyz.y);
-            const float2* __restrict__ Z2 = reinterpret_cast<const float2*>(xyz.z);
-            auto test1 = [&](unsigned j) {
-                const float4 pj = __ldg(pos + j);
-                const float r2 = pair_r2(__fsub_rn(pj.x, pi.x), __fsub_rn(pj.y, pi.y), __fsub_rn(pj.z, pi.z));
-                return (unsigned)(r2 < h2 && r2 != 0.0f);
-            };
-            auto test2 = [&](float2 X, float2 Y, float2 Z) {
-                const float2 dx = __fadd2_rn(X, nx2), dy = __fadd2_rn(Y, ny2), dz = __fadd2_rn(Z, nz2);
-                const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-                return (unsigned)(r2.x < h2 && r2.x != 0.0f) | (unsigned)(r2.y < h2 && r2.y != 0.0f) << 1;
-            };
-            RowWalk walk(c.g, c.wg, cstart, pi.x, pi.y, pi.z);
-            unsigned s0, s1;
-            while (walk.next(s0, s1)) {
-                for (unsigned base = s0; base < s1; base += 32) {
-                    const unsigned e = min(base + 32u, s1);
-                    unsigned m = 0, j = base;
-                    if (j & 1u) m = test1(j++);
-                    const unsigned e2 = e & ~1u;
-                    for (; j + 4 <= e2; j += 4) {
-                        const unsigned k = j >> 1;
-                        const float2 xa = __ldg(X2 + k), ya = __ldg(Y2 + k), za = __ldg(Z2 + k);
-                        const float2 xb = __ldg(X2 + k + 1), yb = __ldg(Y2 + k + 1), zb = __ldg(Z2 + k + 1);
-                        m |= test2(xa, ya, za) << (j - base);
-                        m |= test2(xb, yb, zb) << (j + 2 - base);
-                    }
-                    if (j < e2) {
-                        const unsigned k = j >> 1;
-                        m |= test2(__ldg(X2 + k), __ldg(Y2 + k), __ldg(Z2 + k)) << (j - base);
-                        j += 2;
-                    }
-                    if (j < e) m |= test1(j) << (j - base);
-                    while (m) {
-                        const int t = __ffs(m) - 1;
-                        m &= m - 1u;
-                        pair(base + (unsigned)t);
-                    }
-                }
-            }
-        }
-    }
     const float inv_rho = 1.0f / rho_i;
     float ax = axy.x * inv_rho, ay = axy.y * inv_rho;
     az *= inv_rho;
@@ -723,6 +816,39 @@ __device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
     if (__any_sync(FULL, clamped) && (threadIdx.x & 31) == 0) atomicOr(err, SPH_DEV_CLAMPED);
 }
 
+// The force pass of sorted slot i (i >= n_all: an idle lane), one particle
+// per thread.  Every lane of the warp must call it.
+template <bool COH>
+__device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
+{
+    PairSums s;
+    if (i < a.sc.n_all) {
+        const float4 pi = a.pos[i];
+        if (id_of(pi) >= a.sc.nb_all)
+            s = pair_sums<COH>(a, i, a.sc.c[scene_of(a.sc.pbase, a.sc.S, (unsigned)i)], pi);
+    }
+    integrate<COH>(a, i, s);
+}
+
+// A boid block of the force pass: F_b, a warp per boid, and with the rules'
+// arguments the boid's rules.
+__device__ __forceinline__ void force_boids(const ForceArgs& a, const BoidArgs& r)
+{
+    int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r.bpos_s) {  // with the rules: the boid at sorted boid slot b
+        if (b >= a.sc.nb_all) return;  // whole warps
+        const int s = b, lane = threadIdx.x & 31;
+        b = id_of(r.bpos_s[s]);
+        const float4 f = boid_fb_warp<false>(b, lane, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
+                                             nullptr, a.fb, a.acc);
+        boid_rules_warp(r, a.sc, s, lane, [&](int) { return f; });
+        return;
+    }
+    if (b < a.sc.nb_all && !(a.bmask && !a.bmask[b]))  // uniform per warp
+        boid_fb_warp<false>(b, threadIdx.x & 31, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
+                            a.bmask, a.fb, a.acc);
+}
+
 // The step's force pass.  The first boid_blocks blocks compute F_b, a warp
 // per boid (boid_fb_warp; F_b also goes to acc at the attached slot when
 // acc is given) and, with the rules' arguments, then run the boid's rules;
@@ -733,19 +859,7 @@ __global__ void __launch_bounds__(512)
 k_forces(ForceArgs a, int boid_blocks, BoidArgs r)
 {
     if ((int)blockIdx.x < boid_blocks) {
-        int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (r.bpos_s) {  // with the rules: the boid at sorted boid slot b
-            if (b >= a.sc.nb_all) return;  // whole warps
-            const int s = b, lane = threadIdx.x & 31;
-            b = id_of(r.bpos_s[s]);
-            const float4 f = boid_fb_warp<false>(b, lane, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
-                                                 nullptr, a.fb, a.acc);
-            boid_rules_warp(r, a.sc, s, lane, [&](int) { return f; });
-            return;
-        }
-        if (b < a.sc.nb_all && !(a.bmask && !a.bmask[b]))  // uniform per warp
-            boid_fb_warp<false>(b, threadIdx.x & 31, a.pos, a.vel, a.rho, a.ab, a.start, a.sc, a.slot_of_boid,
-                                a.bmask, a.fb, a.acc);
+        force_boids(a, r);
         return;
     }
     // particles base + lane, base stepping over the fluid blocks' threads; the
@@ -755,6 +869,46 @@ k_forces(ForceArgs a, int boid_blocks, BoidArgs r)
     for (int base = ((int)blockIdx.x - boid_blocks) * (int)blockDim.x; base < a.sc.n_all; base += T)
         force_particle<false>(a, base + (int)threadIdx.x);
 }
+
+// The same with a warp per particle, for launches too small to fill the chip
+// with a thread each: eight particles per block of 256, whose sums the first
+// warp then integrates, a lane each.  A thread waits for each of its 27
+// record loads in turn (15 us at 4,112 particles on 17 SMs); here they are
+// in flight together.
+__global__ void __launch_bounds__(256)
+k_forces_warp(ForceArgs a, int boid_blocks, BoidArgs r)
+{
+    if ((int)blockIdx.x < boid_blocks) {
+        force_boids(a, r);
+        return;
+    }
+    __shared__ PairSums sums[8];
+    __shared__ float4 pairs[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int base = ((int)blockIdx.x - boid_blocks) * 8, i = base + warp;
+    if (i < a.sc.n_all) {
+        const float4 pi = a.pos[i];
+        PairSums s;
+        if (id_of(pi) >= a.sc.nb_all)
+            s = pair_sums_warp(a, i, a.sc.c[scene_of(a.sc.pbase, a.sc.S, (unsigned)i)], pi, pairs[warp]);
+        if (lane == 0) sums[warp] = s;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const bool on = lane < 8 && base + lane < a.sc.n_all;
+        PairSums s;
+        if (on) s = sums[lane];
+        integrate<false>(a, on ? base + lane : a.sc.n_all, s);
+    }
+}
+
+// The fluid blocks take a warp per particle up to this many particles per
+// multiprocessor (12,160 on 152), a thread per particle beyond.  Whole step
+// replayed, us, thread / warp: 2,000 particles 31 / 25 at 26 neighbours,
+// 50 / 29 at 100, 63 / 32 at 250; 8,000 particles 38 / 33, 61 / 46, 96 / 64;
+// 16,000 particles 42 / 48, 74 / 70, 120 / 100; 33,000 64 / 80, 96 / 116,
+// 208 / 230.
+constexpr int FORCES_WARP_PER_SM = 80;
 
 cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* vel, const float* rho, const float2* ab,
                           const float4* prec, const unsigned* start, const uint2* seg, const int* nseg,
@@ -775,7 +929,12 @@ cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* ve
                       slot_of_boid, bmask, fb, acc, touched, infl, pos_next, vel_next, key, rank, count, err};
     BoidArgs r{};
     if (rules) r = *rules;
-    k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks, r);
+    if (fluid && t.use_seg && seg && !list && sc.n_all <= FORCES_WARP_PER_SM * sm_count()) {
+        const int bb = boids ? (sc.nb_all + 7) / 8 : 0;
+        k_forces_warp<<<bb + (sc.n_all + 7) / 8, 256, 0, s>>>(a, bb, r);
+    } else {
+        k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks, r);
+    }
     ++*launches;
     return cudaGetLastError();
 }

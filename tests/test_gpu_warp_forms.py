@@ -1,6 +1,6 @@
-"""The density pass takes a warp per particle in small launches and a thread
-per particle in large ones: a small scene alone against the same scene inside
-a batch too large for the warp form, bit for bit (needs a GB300)."""
+"""The density and force passes take a warp per particle in small launches and a
+thread per particle in large ones: a small scene alone against the same scene
+inside a batch too large for the warp form, bit for bit (needs a GB300)."""
 import numpy as np
 import pytest
 import torch
@@ -32,20 +32,22 @@ CASES = {
 
 
 @pytest.mark.parametrize("name", CASES)
-def test_warp_and_thread_density_agree(name):
+@pytest.mark.parametrize("diagnostics", [False, True])
+def test_warp_and_thread_passes_agree(name, diagnostics):
     n, nb, region, cell, cell_x = CASES[name]
     p, state = _scene(n, nb, region, cell, cell_x, 77)
     # the filler makes the batch too large for the warp form
     per_sm = torch.cuda.get_device_properties(0).multi_processor_count * 108
     pf, fill = _scene(per_sm + 1, 3, (0.9, 0.9, 0.9), 0.5, 0.0, 5)
-    alone = Scene(p, n, nb)
+    alone = Scene(p, n, nb, diagnostics=diagnostics)
     alone.set_state(*state)
-    both = Scene([pf, p], [per_sm + 1, n], [3, nb])
+    both = Scene([pf, p], [per_sm + 1, n], [3, nb], diagnostics=diagnostics)
     both.set_state(*[np.concatenate([a, b]) for a, b in zip(fill, state)])
     for _ in range(2):
         alone.step(1)
         both.step(1)
-        for field in ("rho", "pressure", "nbr_count", "nseg", "ncand"):
+        fields = ("rho", "pressure", "nbr_count", "nseg", "ncand")
+        for field in fields + (("acc", "touched", "influence") if diagnostics else ()):
             a, b = alone.field(field).cpu().numpy(), both.field(field).cpu().numpy()
             # ids: every scene's boids first, then the fluids, scene by scene
             want = np.concatenate([b[3:3 + nb], b[3 + nb + per_sm + 1:]])

@@ -892,8 +892,9 @@ static SoaPos soa_of(const sph_handle* h)
 
 // Keys (if needed), scan, scatter and per-cell sort + gather of the state
 // into the sorted scratch arrays.  consume = true zeroes the counts (in the
-// scan) for the next step's keys.
-static int bin_state(sph_handle* h, cudaStream_t s, bool consume)
+// scan) for the next step's keys.  hide: the attached particles stand at
+// infinity in the SoA copy (every binning writes that copy anew).
+static int bin_state(sph_handle* h, cudaStream_t s, bool consume, bool hide = false)
 {
     if (!h->keys_ready) {
         prof_begin(h, SPH_KIND_KEYS, s);
@@ -911,7 +912,7 @@ static int bin_state(sph_handle* h, cudaStream_t s, bool consume)
     prof_end(h, s);
     prof_begin(h, SPH_KIND_SORT, s);
     CUDA_TRY(h, launch_cellsort_slots(h->cell_start, h->key, h->n, h->tmp, h->tmp_id, h->pos, h->vel, h->pos_s,
-                                      h->vel_s, h->soa, h->n_boid, h->slot_of_boid, s, &h->launches));
+                                      h->vel_s, h->soa, hide, h->n_boid, h->slot_of_boid, s, &h->launches));
     prof_end(h, s);
     if (consume) h->keys_ready = false;
     return SPH_OK;
@@ -933,7 +934,7 @@ static int enqueue_boid_bin(sph_handle* h, cudaStream_t s)
     CUDA_TRY(h, launch_scatter(h->bkey, h->brank, h->bstart, h->n_boid, h->btmp, s, &h->launches));
     // a boid's storage index is its id
     CUDA_TRY(h, launch_cellsort_slots(h->bstart, h->bkey, h->n_boid, h->btmp, h->btmp, h->bpos, h->bvel, h->bpos_s,
-                                      h->bvel_s, nullptr, 0, nullptr, s, &h->launches));
+                                      h->bvel_s, nullptr, false, 0, nullptr, s, &h->launches));
     prof_end(h, s);
     return SPH_OK;
 }
@@ -1470,7 +1471,7 @@ int sph_voxel_density(sph_handle* h, const float* origin, const int* dims, float
     if (!h->has_state) return fail(h, SPH_ERR_STATE, "no state loaded");
     cudaStream_t s = (cudaStream_t)stream;
     h->last_stream = s;
-    int rc = bin_state(h, s, false);
+    int rc = bin_state(h, s, false, true);
     if (rc != SPH_OK) return rc;
     VoxelConst v;
     for (int a = 0; a < 3; ++a) {
@@ -1483,7 +1484,7 @@ int sph_voxel_density(sph_handle* h, const float* origin, const int* dims, float
     v.invR2 = (float)(1.0 / (double)v.R2);
     v.r = particle_radius;
     v.wb = make_bounds(&h->params[0], v.R2, h->params[0].cell_size, cell_x(&h->params[0]));
-    CUDA_TRY(h, launch_voxel_density(h->pos_s, h->cell_start, h->sc, v, phi, counts, s, &h->launches));
+    CUDA_TRY(h, launch_voxel_density(soa_of(h), h->cell_start, h->sc, v, phi, counts, s, &h->launches));
     h->has_step = false;
     return SPH_OK;
 }

@@ -311,7 +311,8 @@ cudaError_t launch_scatter(const unsigned* key, const unsigned* rank, const unsi
 // tmp[s] of its cell, ranks its id tmp_id[s] against the cell's other ids (a
 // contiguous run of tmp_id, read by its threads together) and moves pos/vel
 // to start[c] + rank, also writing x, y, z to the SoA copy (soa, soa_st
-// floats per axis; may be NULL).  The attached particle of boid b records its
+// floats per axis; may be NULL; hide: the attached particles' x there is
+// infinity).  The attached particle of boid b records its
 // sorted slot in slot_of_boid[b].  A cell of n entries costs n reads per
 // entry, which holds for any n: the entries are spread over the chip (a cell
 // of 2,000 boids, the densest of the large tank's, takes 2,000 cached reads).
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(256)
 k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict__ key, int n,
                  const int* __restrict__ tmp, const int* __restrict__ tmp_id, const float4* __restrict__ pos_in,
                  const float4* __restrict__ vel_in, float4* __restrict__ pos_out,
-                 float4* __restrict__ vel_out, float* __restrict__ soa, size_t soa_st, int nb,
+                 float4* __restrict__ vel_out, float* __restrict__ soa, size_t soa_st, int hide, int nb,
                  int* __restrict__ slot_of_boid)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -336,7 +337,7 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
     pos_out[dst] = p;
     vel_out[dst] = vel_in[src];
     if (soa) {
-        soa[dst] = p.x;
+        soa[dst] = hide && id < nb ? INFINITY : p.x;
         soa[soa_st + dst] = p.y;
         soa[2 * soa_st + dst] = p.z;
     }
@@ -345,12 +346,12 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
 
 cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, const int* tmp,
                                   const int* tmp_id, const float4* pos_in, const float4* vel_in,
-                                  float4* pos_out, float4* vel_out, float* soa, int nb, int* slot_of_boid,
-                                  cudaStream_t s, long long* launches)
+                                  float4* pos_out, float4* vel_out, float* soa, bool hide, int nb,
+                                  int* slot_of_boid, cudaStream_t s, long long* launches)
 {
     if (n <= 0) return cudaSuccess;
     k_cellsort_slots<<<(n + 255) / 256, 256, 0, s>>>(start, key, n, tmp, tmp_id, pos_in, vel_in, pos_out, vel_out,
-                                                     soa, soa_stride((size_t)n), nb, slot_of_boid);
+                                                     soa, soa_stride((size_t)n), hide, nb, slot_of_boid);
     ++*launches;
     return cudaGetLastError();
 }

@@ -355,11 +355,12 @@ cudaError_t launch_scatter_ids(const unsigned* key, const unsigned* rank, const 
 // Per-cell sort by particle id + gather, a thread per sorted slot; key holds
 // the cell of every storage slot, n the number of particles.  tmp_id: the
 // ids beside tmp (launch_scatter_ids); soa (may be NULL): the SoA copy of
-// pos_out (soa_stride(n) floats per axis), written as well.
+// pos_out (soa_stride(n) floats per axis), written as well; with hide the
+// particles of ids below nb (the attached ones) stand at infinity in it.
 cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, const int* tmp,
                                   const int* tmp_id, const float4* pos_in, const float4* vel_in,
-                                  float4* pos_out, float4* vel_out, float* soa, int nb, int* slot_of_boid,
-                                  cudaStream_t s, long long* launches);
+                                  float4* pos_out, float4* vel_out, float* soa, bool hide, int nb,
+                                  int* slot_of_boid, cudaStream_t s, long long* launches);
 cudaError_t launch_slot_keys(const unsigned* start, int ncells, unsigned* slot_key, cudaStream_t s,
                              long long* launches);
 
@@ -504,7 +505,9 @@ struct VoxelConst {
     float r;            // particle radius
     WalkBounds wb;      // walk bounds of radius R on the particle grid
 };
-cudaError_t launch_voxel_density(const float4* pos, const unsigned* start, const Scenes& sc, const VoxelConst& v,
+// xyz: the SoA copy with the attached particles at infinity
+// (launch_cellsort_slots, hide).
+cudaError_t launch_voxel_density(const SoaPos& xyz, const unsigned* start, const Scenes& sc, const VoxelConst& v,
                                  float* phi, int* count, cudaStream_t s, long long* launches);
 // Host copies of the generated marching-cubes tables (edge: 256 masks, tri:
 // 256 x 16, -1 terminated); -1 if the generator failed its own checks.

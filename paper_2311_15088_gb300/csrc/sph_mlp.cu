@@ -409,7 +409,7 @@ __global__ void k_cast_weights(const float* __restrict__ P, __nv_bfloat16* __res
 // same order: for each pair of tiles, layer by layer, slot 0 then slot 1,
 // so the MMAs of one slot's next layer run during the epilogue of the
 // other slot's current layer.  The K order and the epilogue arithmetic are
-// those of the per-layer GEMMs that training runs.  Every wait is bounded.
+// those of per-layer GEMMs.  Every wait is bounded.
 namespace fused {
 constexpr int KB_IN = (MLP_IN + BK - 1) / BK;   // 5 K tiles of the input
 constexpr int KB_H = MLP_H / BK;                // 4 K tiles of a hidden layer
@@ -667,8 +667,8 @@ k_mlp_fused(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CU
 // k_train_rows: one CTA per NB batch rows.  The products run transposed,
 // out^T[feature][row] = W[feature][k] . act[row][k]^T, with the weights as
 // the 128-row A operand (two halves of 256 features) and the CTA's rows as
-// the N dimension, because a training batch is small: 2,048 rows make 64
-// CTAs of 32 rows where 128-row tiles make 16.  Seven steps: layers 0 .. 3,
+// the N dimension, because a training batch is small: 2,048 rows make
+// 128 CTAs of 16 rows where 128-row tiles make 16.  Seven steps: layers 0 .. 3,
 // then the backward products through W4, W3, W2.  The rows' activations stay
 // in one shared-memory buffer (K-major 64-column tiles, 128-byte swizzle),
 // each step's epilogue writing its output over its input once the step's
@@ -683,7 +683,8 @@ k_mlp_fused(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CU
 // What bounds it: the chain of seven dependent steps (MMA, epilogue and
 // barrier each), not bandwidth: 0.68 MB of weights per CTA from L2.  A
 // training step of 2,048 rows took 432 us as 26 launches (four 110 us
-// column sums of one thread per column among them).
+// column sums of one thread per column among them); now 21 us here, 10 in
+// k_train_dw, 6 in k_train_update, with the host's part 50.
 namespace train {
 constexpr int STEPS = 7, STAGES = 5, KB_IN = (MLP_IN + BK - 1) / BK, KB_H = MLP_H / BK;
 constexpr uint32_t W_TILE = MLP_H * BK * 2;  // 32 KB: 256 features x 64 BF16
@@ -970,22 +971,30 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
 // 16 SMs.  The last blocks of the first slice sum dT over the batch, the
 // bias gradients: a thread per output adds its row in batch order, one
 // float32 sum (its last bit reaches the next step's activations, so the
-// order is part of the result).  The rows come through the same TMA ring
-// (read straight from memory, a warp's loads of 32 rows were 32 wavefronts
-// each: 21 us for 2,048 rows), so that the chain of additions, 4 cycles
-// each, is what it takes.
+// order is part of the result).  That chain of additions bounds the kernel
+// (the weight tiles alone take 6.6 us for 2,048 rows), so its warp does
+// nothing else: the rows come by TMA from a warp of the copies' own, two
+// blocks of 64 a wait, and the BF16 value is an operand of the addition.  A
+// warp of 32 outputs a block, mixed additions and one wait for two blocks:
+// 13.9 -> 10.2 us (with conversions and a wait a block 14.1, with the mixed
+// additions alone 12.8; read straight from memory, a warp's loads of 32 rows
+// were 32 wavefronts each: 21).
 namespace dw {
-constexpr int NT = 144, STAGES = 4, TILES = 14, BIAS = 7;  // weight tiles, blocks of 128 biases
+constexpr int NT = 144, STAGES = 4, TILES = 14;  // weight tiles
+constexpr int BR = 32, BIAS = 25, BIAS_STAGES = 8;  // bias blocks of 32 outputs: 8 a hidden layer, then the output layer's
 constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = NT * BK * 2, STAGE = A_BYTES + B_BYTES;
 constexpr uint32_t BARS = STAGES * STAGE;
-constexpr uint32_t TOTAL = 1024 + BARS + 8 * (2 * STAGES + 1) + 16;
+constexpr uint32_t BIAS_BYTES = 2 * BR * BK * 2;  // a stage: two blocks of the batch
+constexpr uint32_t TOTAL = 1024 + BARS + 8 * (2 * BIAS_STAGES + 2) + 16;
 constexpr uint32_t TMEM_COLS = 256;
-static_assert(STAGE % 1024 == 0, "operand tiles start on 1024-byte boundaries");
+static_assert(STAGE % 1024 == 0 && BIAS_BYTES % 1024 == 0, "operand tiles start on 1024-byte boundaries");
+static_assert(BIAS_STAGES >= STAGES && BIAS_STAGES * BIAS_BYTES <= BARS, "the biases' ring fits the operands'");
 }  // namespace dw
 
 struct DwMaps {
     CUtensorMap d[4];   // dT of layers 0 .. 3, boxes of 128 rows
     CUtensorMap in[4];  // inT of layers 0 .. 3, boxes of 144 rows
+    CUtensorMap b[4];   // dT of layers 0 .. 3, boxes of 32 rows
 };
 
 __global__ void __launch_bounds__(160)
@@ -1002,71 +1011,72 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
     uint8_t* gbase = smem_raw + (base - raw);
     const uint32_t bars = base + BARS;
     auto full = [&](int s) { return bars + 8u * (uint32_t)s; };
-    auto empty = [&](int s) { return bars + 8u * (uint32_t)(STAGES + s); };
-    const uint32_t done = bars + 8u * (2 * STAGES), tmem_slot = done + 8u;
-    uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(gbase + BARS + 8 * (2 * STAGES + 1));
+    auto empty = [&](int s) { return bars + 8u * (uint32_t)(BIAS_STAGES + s); };
+    const uint32_t done = bars + 8u * (2 * BIAS_STAGES), tmem_slot = done + 8u;
+    uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(gbase + BARS + 8 * (2 * BIAS_STAGES + 1));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const ParamLayout L;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < (bias ? BIAS_STAGES : STAGES); ++s) {
             mbar_init(full(s), 1);
-            mbar_init(empty(s), bias ? 128 : 1);
+            mbar_init(empty(s), bias ? BR : 1);
         }
         mbar_init(done, 1);
         mbar_fence_init();
     }
     if (bias) {
-        // blocks 0 .. 5: halves of the hidden layers, 6: the output layer (the
-        // last block, also where it is the only one)
-        const int blk = BIAS - ((int)gridDim.x - (int)blockIdx.x), l = blk >> 1, m0 = (blk & 1) * BM;
+        // blocks 0 .. 23: the hidden layers, 24: the output layer (the last
+        // block, also where it is the only one)
+        const int blk = BIAS - ((int)gridDim.x - (int)blockIdx.x), l = blk >> 3, m0 = (blk & 7) * BR;
+        const int n = kb_total / 2;  // the batch is a multiple of two blocks
         __syncthreads();
         if (warp == 4) {  // the copies' own warp: in a summing warp they would hold up its chain
             if (lane == 0) {
                 int i = 0;
-                for (; i < kb_total; ++i) {
-                    const int st = i % STAGES;
-                    if (i >= STAGES && !mbar_wait(empty(st), (uint32_t)((i / STAGES) - 1) & 1u, err)) break;
-                    mbar_expect_tx(full(st), A_BYTES);
-                    tma_load_2d(&maps.d[l], full(st), base + st * STAGE, i * BK, m0);
+                for (; i < n; ++i) {
+                    const int st = i % BIAS_STAGES;
+                    if (i >= BIAS_STAGES && !mbar_wait(empty(st), (uint32_t)((i / BIAS_STAGES) - 1) & 1u, err)) break;
+                    mbar_expect_tx(full(st), BIAS_BYTES);
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_2d(&maps.b[l], full(st), base + st * BIAS_BYTES + h * (BIAS_BYTES / 2), (2 * i + h) * BK, m0);
                 }
-                if (i < kb_total)  // let the copies in flight land before the CTA goes away
-                    for (int q = max(0, i - STAGES); q < i; ++q)
-                        mbar_wait(full(q % STAGES), (uint32_t)(q / STAGES) & 1u, err);
+                if (i < n)  // let the copies in flight land before the CTA goes away
+                    for (int q = max(0, i - BIAS_STAGES); q < i; ++q)
+                        mbar_wait(full(q % BIAS_STAGES), (uint32_t)(q / BIAS_STAGES) & 1u, err);
             }
             return;
         }
+        if (warp) return;
         // a row's 64 values of a block are loaded while the block before is added
         uint4 v[2][BK / 8];
         float s = 0.f;
-        auto fetch = [&](int i, uint4 (&to)[BK / 8]) {
-            const int st = i % STAGES;
-            if (!mbar_wait(full(st), (uint32_t)(i / STAGES) & 1u, err)) return false;
-            const uint8_t* row = gbase + st * STAGE;
+        auto wait = [&](int i) { return mbar_wait(full(i % BIAS_STAGES), (uint32_t)(i / BIAS_STAGES) & 1u, err); };
+        auto fetch = [&](int i, int h) {
+            const uint8_t* row = gbase + (i % BIAS_STAGES) * BIAS_BYTES + h * (BIAS_BYTES / 2);
 #pragma unroll
-            for (int c = 0; c < BK / 8; ++c)
-                to[c] = *reinterpret_cast<const uint4*>(row + sw128_offset((int)threadIdx.x, 8 * c));
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty(st)) : "memory");
-            return true;
+            for (int c = 0; c < BK / 8; ++c) v[h][c] = *reinterpret_cast<const uint4*>(row + sw128_offset(lane, 8 * c));
         };
         auto sum = [&](const uint4 (&from)[BK / 8]) {
 #pragma unroll
             for (int c = 0; c < BK / 8; ++c) {
                 const uint32_t w[4] = {from[c].x, from[c].y, from[c].z, from[c].w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {  // BF16 -> FP32 is the high half of the word
-                    s = __fadd_rn(s, __uint_as_float(w[j] << 16));
-                    s = __fadd_rn(s, __uint_as_float(w[j] & 0xffff0000u));
-                }
+                for (int j = 0; j < 4; ++j)  // float32 + BF16, rounded once
+                    asm("{.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %0, h, %0;}"
+                        : "+f"(s)
+                        : "r"(w[j]));
             }
         };
-        bool ok = fetch(0, v[0]);
-        for (int i = 0; ok && i < kb_total; i += 2) {  // an even number of blocks
-            ok = fetch(i + 1, v[1]);
+        bool ok = wait(0);
+        if (ok) fetch(0, 0);
+        for (int i = 0; ok && i < n; ++i) {
+            fetch(i, 1);
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty(i % BIAS_STAGES)) : "memory");
             sum(v[0]);
-            if (ok && i + 2 < kb_total) ok = fetch(i + 2, v[0]);
+            if (i + 1 < n && (ok = wait(i + 1))) fetch(i + 1, 0);
             sum(v[1]);
         }
-        const int f = m0 + (int)threadIdx.x;
+        const int f = m0 + lane;
         if (ok && f < L.out[l])  // the other slices hold zeros
             for (int k = 0; k < (int)gridDim.y; ++k) part[(size_t)k * SPH_MLP_PARAMS + L.b[l] + f] = k ? 0.0f : s;
         return;
@@ -1334,6 +1344,7 @@ static int train_maps(sph_mlp* m)
     for (int l = 0; l < 4; ++l) {
         MLP_TRY(m, make_map(&m->dmaps.d[l], l < 3 ? m->DT[l] : m->DYT, L.out[l], m->max_batch, m->max_batch, BM));
         MLP_TRY(m, make_map(&m->dmaps.in[l], l ? m->HT[l - 1] : m->XT, L.in[l], m->max_batch, m->max_batch, dw::NT));
+        MLP_TRY(m, make_map(&m->dmaps.b[l], l < 3 ? m->DT[l] : m->DYT, L.out[l], m->max_batch, m->max_batch, dw::BR));
     }
     m->maps_ready = true;
     return SPH_OK;

@@ -948,8 +948,8 @@ def run_ours(a):
     n_all = nf + nb
     passes = {k: {"ms_per_step": ms / max(cnt, 1), "launch_groups": cnt} for k, (ms, cnt) in prof.items() if cnt}
     if nb:
-        passes["note"] = ("boid_bin and boid_rules (F_b + rules) run on the step's side stream alongside the "
-                          "fluid passes: their times are spans that overlap density and forces")
+        passes["note"] = ("boid_bin runs on the step's side stream alongside the fluid's binning and density pass: "
+                          "its time is a span that overlaps them; F_b and the boid rules run in the force launch")
     f_ms = passes["forces"]["ms_per_step"]
     d_ms = passes["density"]["ms_per_step"]
     stencil = STENCIL_CAND_PER_NBR * pairs

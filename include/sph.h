@@ -446,7 +446,9 @@ long long sph_launch_count(sph_handle* h);
  * (exclusive scan of the cell counts), SPH_KIND_SCATTER, SPH_KIND_SORT
  * (per-cell sort + gather), SPH_KIND_DENSITY, SPH_KIND_FORCES (pair forces
  * + integration + next keys), SPH_KIND_BOID_BIN (boid-grid binning),
- * SPH_KIND_BOID_RULES, SPH_KIND_LISTS, SPH_KIND_FEATURES, SPH_KIND_PIPELINE
+ * SPH_KIND_BOID_RULES (the rules where they are a launch of their own: after
+ * the fused pipeline; otherwise they run in the force pass's launch and its
+ * time holds theirs), SPH_KIND_LISTS, SPH_KIND_FEATURES, SPH_KIND_PIPELINE
  * (SPH_NUM_KINDS kinds).  sph_profile_enable(h, n) creates a host-side pool
  * of 2n events (n = 0 disables and frees it); while enabled, each pass of
  * sph_step is bracketed by two events recorded on the step's stream, up to
@@ -644,9 +646,10 @@ int sph_voxel_density(sph_handle* h, const float origin[3], const int dims[3], f
  * order; triangles wind so that their right-hand normal points to the side
  * below iso.  At most max_tris are written; *ntri (a device unsigned)
  * receives the total, which may exceed max_tris (saturated at 0xfffffffe).
- * Three launches: the triangle counts of tiles of 1,024 cubes, one scan of
- * the tile totals, then each tile's triangles from its offset, spread
- * evenly over the tile's threads.  workspace: device memory of
+ * Two launches: the triangle counts of tiles of 1,024 cubes, then each
+ * tile's triangles from its offset (the totals of the tiles before it),
+ * spread evenly over the tile's threads; beyond 8,192 tiles a third, between
+ * them, scans the tile totals.  workspace: device memory of
  * sph_mc_workspace_size bytes, 256-byte aligned, owned by the caller.
  * The first call on a device copies the tables to its memory
  * (synchronously); make it before any stream capture.  Errors: SPH_ERR_ARG

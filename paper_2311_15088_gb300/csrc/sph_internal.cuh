@@ -515,8 +515,8 @@ int mc_tables_host(unsigned short* edge, signed char* tri);
 // Copy the tables to the current device's constant memory (once per device).
 cudaError_t mc_upload_tables();
 // Tiles of consecutive cubes: per-tile counts (each cube's case byte kept
-// in cases[ncubes]), one scan of the tile totals, then the triangles from
-// each tile's offset (three launches).  tile_count and tile_off hold
+// in cases[ncubes]), then the triangles from each tile's offset (two
+// launches; beyond 8,192 tiles a scan of the totals between them).  tile_count and tile_off hold
 // mc_tiles(ncubes) words; *total receives the triangle count.
 long long mc_tiles(long long ncubes);
 cudaError_t launch_marching_cubes(const float* phi, const int dims[3], const float origin[3], float spacing,

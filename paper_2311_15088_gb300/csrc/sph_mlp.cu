@@ -1,17 +1,18 @@
 // sph_mlp.cu -- the boid-force surrogate: a 272 -> 256 -> 256 -> 256 -> 16
-// MLP (exact-erf GELU) whose inference and training GEMMs run on the
-// tensor cores (tcgen05.mma kind::f16: BF16 operands staged by TMA, FP32
-// accumulators in tensor memory), with Adam on FP32 master weights.
+// MLP (exact-erf GELU) whose inference (k_mlp_fused; small batches
+// k_train_rows) and training (k_train_*) run on the tensor cores
+// (tcgen05.mma kind::f16: BF16 operands staged by TMA, FP32 accumulators in
+// tensor memory), with Adam on FP32 master weights.
 //
 // The surrogate is not in the paper; it predicts the fluid force the SPH
 // coupling of section "Boid Motion and Agent Fluid Interaction" puts on a
 // boid (F_b in v_b += sph_factor dt F_b) from the flow around the boid.
 //
 // Layout: a layer's weight W is [out][in] (K-major for the B operand of the
-// forward GEMM) with a transposed BF16 copy W^T [in][out] for the backward
-// GEMM; activations are [batch][features] with transposed copies
-// [features][batch] for the weight-gradient GEMMs (which contract over the
-// batch).  Every GEMM is C[M][N] = A[M][K] . B[N][K]^T with both operands
+// forward products) with a transposed BF16 copy W^T [in][out] for the
+// backward ones; activations are [batch][features] with transposed copies
+// [features][batch] for the weight gradients (which contract over the
+// batch).  Every product is C[M][N] = A[M][K] . B[N][K]^T with both operands
 // K-major.
 #include <cudaTypedefs.h>
 #include <math.h>

@@ -1,6 +1,6 @@
-// sph_bin.cu -- uniform-grid binning of the step: cell keys with a
-// warp-aggregated histogram, exclusive scan of the cell counts, scatter and
-// a per-cell sort by particle id fused with the gather of the SoA state.
+// sph_bin.cu -- uniform-grid binning of the step: cell keys with the
+// cells' histogram, exclusive scan of the cell counts, scatter and a per-cell
+// sort by particle id fused with the gather of the SoA state.
 //
 // Paper: section "Neighborhood Search" (get_cell, hash) and section
 // "Neighbor Search with Sorting" (set_particle_count, prefix sum,
@@ -33,8 +33,7 @@ k_keys(const float4* __restrict__ pos, int n, GridDesc g, Box box, unsigned* __r
         key[i] = k;
         clamped = outside_box(box, p.x, p.y, p.z);
     }
-    unsigned r = agg_increment(count, k, active);
-    if (active) rank[i] = r;
+    if (active) rank[i] = count_in_cell(count, k);
     if (__any_sync(FULL, clamped) && (threadIdx.x & 31) == 0) atomicOr(err, SPH_DEV_CLAMPED);
 }
 
@@ -72,8 +71,7 @@ k_scene_keys(const float4* __restrict__ pos, Scenes sc, unsigned* __restrict__ k
         // boid-attached particles follow their boids, which may leave the tank
         clamped = id_of(p) >= sc.nb_all && outside_box(c, p.x, p.y, p.z);
     }
-    unsigned r = agg_increment(count, k, active);
-    if (active) rank[i] = r;
+    if (active) rank[i] = count_in_cell(count, k);
     if (__any_sync(FULL, clamped) && (threadIdx.x & 31) == 0) atomicOr(err, SPH_DEV_CLAMPED);
 }
 

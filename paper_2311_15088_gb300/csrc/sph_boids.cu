@@ -22,17 +22,14 @@ k_boid_keys(const float4* __restrict__ bpos, Scenes sc, unsigned* __restrict__ b
             unsigned* __restrict__ brank, unsigned* __restrict__ bcount)
 {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
-    bool active = b < sc.nb_all;
-    unsigned k = 0;
     bool clamped = false;
-    if (active) {
+    if (b < sc.nb_all) {
         const StepConst& c = sc.c[scene_of(sc.bbase, sc.S, (unsigned)b)];
         float4 p = bpos[b];
-        k = (unsigned)c.cb_base + cell_key(c.gb, p.x, p.y, p.z, &clamped);
+        const unsigned k = (unsigned)c.cb_base + cell_key(c.gb, p.x, p.y, p.z, &clamped);
         bkey[b] = k;
+        brank[b] = count_in_cell(bcount, k);
     }
-    unsigned r = agg_increment(bcount, k, active);
-    if (active) brank[b] = r;
 }
 
 cudaError_t launch_boid_keys(const float4* bpos, const Scenes& sc, unsigned* bkey, unsigned* brank,

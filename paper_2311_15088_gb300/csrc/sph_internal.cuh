@@ -113,23 +113,12 @@ __device__ __forceinline__ float pair_r2(float dx, float dy, float dz)
     return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
 }
 
-// Warp-aggregated counter increment: lanes with the same key share one
-// atomicAdd; returns each lane's slot.  Every lane of the warp must call it.
-__device__ __forceinline__ unsigned agg_increment(unsigned* count, unsigned k, bool active)
-{
-    unsigned act = __ballot_sync(FULL, active);
-    unsigned slot = 0;
-    if (active) {
-        unsigned peers = __match_any_sync(act, k);
-        int lane = threadIdx.x & 31;
-        int leader = __ffs(peers) - 1;
-        unsigned base = 0;
-        if (lane == leader) base = atomicAdd(&count[k], (unsigned)__popc(peers));
-        base = __shfl_sync(peers, base, leader);
-        slot = base + (unsigned)__popc(peers & ((1u << lane) - 1u));
-    }
-    return slot;
-}
+// Count a particle in cell k; returns its place among the cell's arrivals
+// (any order: the per-cell sort is by id).  An atomic per particle: with the
+// lanes of equal keys found by a warp match and sharing one, binning the
+// loaded 2M-particle tank's keys took 46 us and the 4.2M particles of 256
+// tanks 100; now 24 and 44.
+__device__ __forceinline__ unsigned count_in_cell(unsigned* count, unsigned k) { return atomicAdd(count + k, 1u); }
 
 __device__ __forceinline__ int id_of(const float4& p) { return __float_as_int(p.w); }
 

@@ -745,7 +745,7 @@ __device__ __forceinline__ PairSums pair_sums_warp(const ForceArgs& a, int i, co
 // next step's cell keys.  acc, touched and infl (the diagnostic fields) are
 // written only when given (all three or none); attached particles then
 // record touched = 0 and influence = 0 (attached pairs are excluded).  Every
-// lane of the warp must call it (warp-aggregated counting).
+// lane of the warp must call it (one report of a clamped position).
 template <bool COH>
 __device__ __forceinline__ void integrate(const ForceArgs& a, int i, const PairSums& s)
 {
@@ -776,7 +776,6 @@ __device__ __forceinline__ void integrate(const ForceArgs& a, int i, const PairS
     az *= inv_rho;
     const float bx = bxy.x, by = bxy.y;
 
-    unsigned k_next = 0;
     if (active && touched) {
         touched[i] = touch;
         infl[i] = make_float4(bx * inv_rho, by * inv_rho, bz * inv_rho, 0.0f);
@@ -807,12 +806,11 @@ __device__ __forceinline__ void integrate(const ForceArgs& a, int i, const PairS
         pos_next[i] = make_float4(x[0], x[1], x[2], pi.w);
         vel_next[i] = make_float4(v[0], v[1], v[2], 0.0f);
         bool cl = false;
-        k_next = (unsigned)c.c_base + cell_key(c.g, x[0], x[1], x[2], &cl);
+        const unsigned k_next = (unsigned)c.c_base + cell_key(c.g, x[0], x[1], x[2], &cl);
         key[i] = k_next;
+        rank[i] = count_in_cell(count, k_next);
         clamped = outside_box(c, x[0], x[1], x[2]);  // NaN only: the walls keep x in the box
     }
-    unsigned r = agg_increment(count, k_next, fluid);
-    if (fluid) rank[i] = r;
     if (__any_sync(FULL, clamped) && (threadIdx.x & 31) == 0) atomicOr(err, SPH_DEV_CLAMPED);
 }
 
@@ -864,7 +862,7 @@ k_forces(ForceArgs a, int boid_blocks, BoidArgs r)
     }
     // particles base + lane, base stepping over the fluid blocks' threads; the
     // trip count is the block's, so every lane of a warp takes part in each
-    // call (force_particle's warp-aggregated count)
+    // call (force_particle's one report per warp)
     const int T = ((int)gridDim.x - boid_blocks) * (int)blockDim.x;
     for (int base = ((int)blockIdx.x - boid_blocks) * (int)blockDim.x; base < a.sc.n_all; base += T)
         force_particle<false>(a, base + (int)threadIdx.x);

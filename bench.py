@@ -90,13 +90,14 @@ BYTES_PER_CELL_SCAN = 12
 # (sph_physics.cu, sph_internal.cuh) it was taken on; null once they moved.
 # Capture: the launch list (gpu__time_duration, dram__bytes_read/write, one
 # pass) of `bench.py --steps 20 --warmup 3 --no-cpu-baseline --e2e-steps 2
-# --no-batch --no-surrogate --no-surface`, mean over the 21 launches of the
-# timed steps after 200 settling steps (k_forces: the fluid launches).
+# --no-batch --no-surrogate --no-surface`, mean over the 24 launches of the
+# warm-up, timed and end-to-end steps after 200 settling steps (k_forces: the
+# fluid particles, F_b and the boid rules in one launch).
 KERNEL_TRAFFIC = {
-    "k_forces": {"bytes": 720.4e6, "read": 643.0e6, "write": 77.4e6,
-                 "source_sha256": "6b796b8c825557b856e8bbf3bfed9d904664eaa34e59dceed01518a5c17eb9c8"},
-    "k_density": {"bytes": 864.2e6, "read": 289.4e6, "write": 574.8e6,
-                  "source_sha256": "6b796b8c825557b856e8bbf3bfed9d904664eaa34e59dceed01518a5c17eb9c8"},
+    "k_forces": {"bytes": 739.9e6, "read": 656.0e6, "write": 83.9e6,
+                 "source_sha256": "4151dfe0332fedba9ed8b49b1f5aaf87e9f4959196a7d5773f5397b11e05c61a"},
+    "k_density": {"bytes": 865.8e6, "read": 290.3e6, "write": 575.5e6,
+                  "source_sha256": "4151dfe0332fedba9ed8b49b1f5aaf87e9f4959196a7d5773f5397b11e05c61a"},
 }
 
 

@@ -16,6 +16,8 @@
 // z, y order, x ascending, each row clipped to the sphere), so its float32
 // sums have a fixed order that depends only on the state.  Neighbouring
 // threads share cells, so the candidate loads are served by L1.
+#include <algorithm>
+
 #include "sph_boids.cuh"
 
 namespace sphk {
@@ -830,9 +832,9 @@ __device__ __forceinline__ void force_particle(const ForceArgs& a, int i)
 
 // A boid block of the force pass: F_b, a warp per boid, and with the rules'
 // arguments the boid's rules.
-__device__ __forceinline__ void force_boids(const ForceArgs& a, const BoidArgs& r)
+__device__ __forceinline__ void force_boids(const ForceArgs& a, const BoidArgs& r, int block)
 {
-    int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    int b = block * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
     if (r.bpos_s) {  // with the rules: the boid at sorted boid slot b
         if (b >= a.sc.nb_all) return;  // whole warps
         const int s = b, lane = threadIdx.x & 31;
@@ -847,24 +849,30 @@ __device__ __forceinline__ void force_boids(const ForceArgs& a, const BoidArgs& 
                             a.bmask, a.fb, a.acc);
 }
 
-// The step's force pass.  The first boid_blocks blocks compute F_b, a warp
+// The step's force pass.  boid_blocks blocks, every boid_step-th from the
+// first on, compute F_b, a warp
 // per boid (boid_fb_warp; F_b also goes to acc at the attached slot when
 // acc is given) and, with the rules' arguments, then run the boid's rules;
 // they come first in the grid so that these latency-bound warps run
-// alongside the fluid blocks.  The remaining blocks (possibly
-// none) take a particle per thread (force_particle).
+// alongside the fluid blocks, and where they alone would fill the chip for
+// several waves, between the fluid blocks: the 2M-particle tank with 16,384
+// boids 3.298 -> 3.278 ms a step, 256 tanks 5.82 -> 5.80 a pass; the column's
+// 1,024 boids, which fit at once, 1.084 -> 1.095 if spread.  The remaining
+// blocks (possibly none) take a particle per thread (force_particle).
 __global__ void __launch_bounds__(512)
-k_forces(ForceArgs a, int boid_blocks, BoidArgs r)
+k_forces(ForceArgs a, int boid_blocks, int boid_step, BoidArgs r)
 {
-    if ((int)blockIdx.x < boid_blocks) {
-        force_boids(a, r);
+    const int block = (int)blockIdx.x, group = block / boid_step;
+    if (group < boid_blocks && block == group * boid_step) {
+        force_boids(a, r, group);
         return;
     }
+    const int fluid_block = block - min(group + 1, boid_blocks);
     // particles base + lane, base stepping over the fluid blocks' threads; the
     // trip count is the block's, so every lane of a warp takes part in each
     // call (force_particle's one report per warp)
     const int T = ((int)gridDim.x - boid_blocks) * (int)blockDim.x;
-    for (int base = ((int)blockIdx.x - boid_blocks) * (int)blockDim.x; base < a.sc.n_all; base += T)
+    for (int base = fluid_block * (int)blockDim.x; base < a.sc.n_all; base += T)
         force_particle<false>(a, base + (int)threadIdx.x);
 }
 
@@ -877,7 +885,7 @@ __global__ void __launch_bounds__(256)
 k_forces_warp(ForceArgs a, int boid_blocks, BoidArgs r)
 {
     if ((int)blockIdx.x < boid_blocks) {
-        force_boids(a, r);
+        force_boids(a, r, (int)blockIdx.x);
         return;
     }
     __shared__ PairSums sums[8];
@@ -931,7 +939,11 @@ cudaError_t launch_forces(const float4* pos, const SoaPos& xyz, const float4* ve
         const int bb = boids ? (sc.nb_all + 7) / 8 : 0;
         k_forces_warp<<<bb + (sc.n_all + 7) / 8, 256, 0, s>>>(a, bb, r);
     } else {
-        k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks, r);
+        // more boid warps than the chip holds at once (32 an SM): every fourth
+        // block, or as sparse as the fluid blocks allow
+        const bool spread = boid_blocks * warps > 32 * sm_count();
+        const int step = spread ? std::min(4, (boid_blocks + fluid_blocks) / boid_blocks) : 1;
+        k_forces<<<boid_blocks + fluid_blocks, t.block, 0, s>>>(a, boid_blocks, step, r);
     }
     ++*launches;
     return cudaGetLastError();

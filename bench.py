@@ -94,10 +94,10 @@ BYTES_PER_CELL_SCAN = 12
 # warm-up, timed and end-to-end steps after 200 settling steps (k_forces: the
 # fluid particles, F_b and the boid rules in one launch).
 KERNEL_TRAFFIC = {
-    "k_forces": {"bytes": 739.9e6, "read": 656.0e6, "write": 83.9e6,
-                 "source_sha256": "4151dfe0332fedba9ed8b49b1f5aaf87e9f4959196a7d5773f5397b11e05c61a"},
+    "k_forces": {"bytes": 742.6e6, "read": 653.3e6, "write": 89.3e6,
+                 "source_sha256": "9b79df2903c2b3808b9b5c212a228f966328cd940ce5c70c1da2e20df8ec1065"},
     "k_density": {"bytes": 865.8e6, "read": 290.3e6, "write": 575.5e6,
-                  "source_sha256": "4151dfe0332fedba9ed8b49b1f5aaf87e9f4959196a7d5773f5397b11e05c61a"},
+                  "source_sha256": "9b79df2903c2b3808b9b5c212a228f966328cd940ce5c70c1da2e20df8ec1065"},
 }
 
 

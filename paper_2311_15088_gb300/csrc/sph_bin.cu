@@ -311,9 +311,18 @@ cudaError_t launch_scatter(const unsigned* key, const unsigned* rank, const unsi
 // to start[c] + rank, also writing x, y, z to the SoA copy (soa, soa_st
 // floats per axis; may be NULL; hide: the attached particles' x there is
 // infinity).  The attached particle of boid b records its
-// sorted slot in slot_of_boid[b].  A cell of n entries costs n reads per
-// entry, which holds for any n: the entries are spread over the chip (a cell
-// of 2,000 boids, the densest of the large tank's, takes 2,000 cached reads).
+// sorted slot in slot_of_boid[b].  A cell of n entries costs n comparisons per
+// entry; the entries are spread over the chip.  Read id by id, a crowded
+// cell's pass waited for every 128-byte line in turn (its warps reach each new
+// line together), so a warp passes the ids of a cell of more than SORT_STREAM
+// entries through shared memory, 32 at a time, the next 64 on their way
+// meanwhile.  One cell of 2,000, 16,000 and 40,000 entries, us: by a block's
+// bitonic sort (which ranked the last by counting) 34, 213 and 66,000, read id
+// by id 38, 265 and 661, now 20, 114 and 378; the large tank's boids 26 -> 17.  Lines of 32 to 256 entries give the same times.  The
+// shared memory is kept small: with 128 ids a warp the tank's particles, which
+// need none of it, took 59 instead of 58 (57 without the branch).
+constexpr int SORT_STREAM = 128;
+
 __global__ void __launch_bounds__(256)
 k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict__ key, int n,
                  const int* __restrict__ tmp, const int* __restrict__ tmp_id, const float4* __restrict__ pos_in,
@@ -321,15 +330,48 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
                  float4* __restrict__ vel_out, float* __restrict__ soa, size_t soa_st, int hide, int nb,
                  int* __restrict__ slot_of_boid)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const int src = tmp[s];
-    const unsigned c = key[src];
-    const unsigned s0 = start[c];
-    const int nc = (int)(start[c + 1] - s0);
-    const int id = tmp_id[s];
+    __shared__ __align__(16) int s_ids[256 / 32][32];
+    const int s = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool active = s < n;
+    int src = 0, nc = 0, id = 0;
+    unsigned s0 = 0;
+    if (active) {
+        src = tmp[s];
+        const unsigned c = key[src];
+        s0 = start[c];
+        nc = (int)(start[c + 1] - s0);
+        id = tmp_id[s];
+    }
+    const bool crowded = nc > SORT_STREAM;
     int r = 0;
-    for (int k = 0; k < nc; ++k) r += __ldg(tmp_id + s0 + k) < id;
+    if (!crowded)
+        for (int k = 0; k < nc; ++k) r += __ldg(tmp_id + s0 + k) < id;
+    // the crowded cells of the warp's slots, one after another
+    for (unsigned todo = __ballot_sync(FULL, crowded); todo;) {
+        const int lead = __ffs((int)todo) - 1;
+        const unsigned c0 = __shfl_sync(FULL, s0, lead), c1 = c0 + (unsigned)__shfl_sync(FULL, nc, lead);
+        int* ids = s_ids[threadIdx.x >> 5];
+        // past the cell: above every id
+        auto fetch = [&](unsigned k) { return k < c1 ? __ldg(tmp_id + k) : 0x7fffffff; };
+        int below = 0;
+        int next = fetch(c0 + lane), next2 = fetch(c0 + 32 + lane);
+        for (unsigned k = c0; k < c1; k += 32) {
+            __syncwarp();  // the 32 before are read
+            ids[lane] = next;
+            __syncwarp();
+            next = next2;
+            next2 = fetch(k + 64 + lane);
+#pragma unroll
+            for (int q = 0; q < 32; q += 4) {
+                const int4 o = *reinterpret_cast<const int4*>(ids + q);
+                below += (o.x < id) + (o.y < id) + (o.z < id) + (o.w < id);
+            }
+        }
+        const bool mine = crowded && s0 == c0;
+        if (mine) r = below;
+        todo &= ~__ballot_sync(FULL, mine);
+    }
+    if (!active) return;
     const unsigned dst = s0 + (unsigned)r;
     const float4 p = pos_in[src];
     pos_out[dst] = p;

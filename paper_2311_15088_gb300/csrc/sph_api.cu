@@ -893,7 +893,7 @@ static SoaPos soa_of(const sph_handle* h)
 // Keys (if needed), scan, scatter and per-cell sort + gather of the state
 // into the sorted scratch arrays.  consume = true zeroes the counts (in the
 // scan) for the next step's keys.  hide: the attached particles stand at
-// infinity in the SoA copy (every binning writes that copy anew).
+// HIDDEN in the SoA copy (every binning writes that copy anew).
 static int bin_state(sph_handle* h, cudaStream_t s, bool consume, bool hide = false)
 {
     if (!h->keys_ready) {
@@ -1483,7 +1483,10 @@ int sph_voxel_density(sph_handle* h, const float* origin, const int* dims, float
     v.R2 = radius * radius;
     v.invR2 = (float)(1.0 / (double)v.R2);
     v.r = particle_radius;
-    v.wb = make_bounds(&h->params[0], v.R2, h->params[0].cell_size, cell_x(&h->params[0]));
+    const sph_params* p = &h->params[0];
+    v.wb = make_bounds(p, v.R2, p->cell_size, cell_x(p));
+    // cells of a row times the particles a cell holds: a mean chord of 4/3 R, widened to whole cells
+    v.row = p->rho0 / p->mass * p->cell_size * p->cell_size * (4.0f / 3.0f * radius + cell_x(p));
     CUDA_TRY(h, launch_voxel_density(soa_of(h), h->cell_start, h->sc, v, phi, counts, s, &h->launches));
     h->has_step = false;
     return SPH_OK;

@@ -309,9 +309,10 @@ cudaError_t launch_scatter(const unsigned* key, const unsigned* rank, const unsi
 // tmp[s] of its cell, ranks its id tmp_id[s] against the cell's other ids (a
 // contiguous run of tmp_id, read by its threads together) and moves pos/vel
 // to start[c] + rank, also writing x, y, z to the SoA copy (soa, soa_st
-// floats per axis; may be NULL; hide: the attached particles' x there is
-// infinity).  The attached particle of boid b records its
-// sorted slot in slot_of_boid[b].  A cell of n entries costs n comparisons per
+// floats per axis; may be NULL; hide: attached particles and positions that
+// are not finite stand at HIDDEN there; the unpaired slot behind an odd number
+// of particles is finite).  The attached particle of boid b records its sorted
+// slot in slot_of_boid[b].  A cell of n entries costs n comparisons per
 // entry; the entries are spread over the chip.  Read id by id, a crowded
 // cell's pass waited for every 128-byte line in turn (its warps reach each new
 // line together), so a warp passes the ids of a cell of more than SORT_STREAM
@@ -377,9 +378,11 @@ k_cellsort_slots(const unsigned* __restrict__ start, const unsigned* __restrict_
     pos_out[dst] = p;
     vel_out[dst] = vel_in[src];
     if (soa) {
-        soa[dst] = hide && id < nb ? INFINITY : p.x;
-        soa[soa_st + dst] = p.y;
-        soa[2 * soa_st + dst] = p.z;
+        const bool away = hide && (id < nb || !(fabsf(p.x) < HIDDEN && fabsf(p.y) < HIDDEN && fabsf(p.z) < HIDDEN));
+        soa[dst] = away ? HIDDEN : p.x;
+        soa[soa_st + dst] = away ? 0.0f : p.y;
+        soa[2 * soa_st + dst] = away ? 0.0f : p.z;
+        if (s == n - 1 && (n & 1)) soa[n] = soa[soa_st + n] = soa[2 * soa_st + n] = 0.0f;
     }
     if (id < nb && slot_of_boid) slot_of_boid[id] = (int)dst;
 }

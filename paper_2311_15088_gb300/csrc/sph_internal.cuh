@@ -345,7 +345,8 @@ cudaError_t launch_scatter_ids(const unsigned* key, const unsigned* rank, const 
 // the cell of every storage slot, n the number of particles.  tmp_id: the
 // ids beside tmp (launch_scatter_ids); soa (may be NULL): the SoA copy of
 // pos_out (soa_stride(n) floats per axis), written as well; with hide the
-// particles of ids below nb (the attached ones) stand at infinity in it.
+// particles of ids below nb (the attached ones) and those of a position that
+// is not finite stand at HIDDEN in it.
 cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, int n, const int* tmp,
                                   const int* tmp_id, const float4* pos_in, const float4* vel_in,
                                   float4* pos_out, float4* vel_out, float* soa, bool hide, int nb,
@@ -371,6 +372,10 @@ struct SoaPos {
 };
 // Elements per axis of the SoA copy of n positions (even).
 __host__ __device__ inline size_t soa_stride(size_t n) { return (n + 1) & ~(size_t)1; }
+
+// The x of what a pass over the SoA copy shall not meet: finite, with an
+// infinite square (no distance from it is below a radius, and 0 times it is 0).
+constexpr float HIDDEN = 1e30f;
 
 // Launch shape of the neighbour passes (chosen by the autotuner; results do
 // not depend on it).
@@ -493,9 +498,10 @@ struct VoxelConst {
     float R, R2, invR2; // neighbourhood radius, fl(R R), fl(1 / R2)
     float r;            // particle radius
     WalkBounds wb;      // walk bounds of radius R on the particle grid
+    float row;          // candidates of a walked row at rest density
 };
-// xyz: the SoA copy with the attached particles at infinity
-// (launch_cellsort_slots, hide).
+// xyz: the SoA copy with the attached particles hidden (launch_cellsort_slots,
+// hide).
 cudaError_t launch_voxel_density(const SoaPos& xyz, const unsigned* start, const Scenes& sc, const VoxelConst& v,
                                  float* phi, int* count, cudaStream_t s, long long* launches);
 // Host copies of the generated marching-cubes tables (edge: 256 masks, tri:

@@ -244,12 +244,21 @@ cudaError_t mc_upload_tables()
 // --------------------------------------------------------- voxel density
 
 // A thread per corner; its candidates come by slot pairs (2k, 2k + 1) from
-// the SoA copy, in which the attached particles stand at infinity (they are
-// no fluid; a candidate at infinity is none of a corner's neighbours), tested
-// and summed side by side with packed float32x2 operations: the even and the
-// odd slots' sums are kept apart and added at the end.  Bound by instruction
-// issue: candidate by candidate from the 16-byte positions, with the id
-// tested, the 1.6M corners of the 2M-particle tank took 375 us, now 329.
+// the SoA copy, in which what is no fluid stands at HIDDEN (none of a corner's
+// neighbours), tested and summed side by side with packed float32x2
+// operations: the even and the odd slots' sums are kept apart and added at the
+// end.  A row's first and last pair may hold a slot of the next row, set to
+// HIDDEN as well (a lone slot read by itself cost as much as a pair).  Bound
+// by instruction issue.  LONG: two pairs in flight an iteration, which long
+// rows repay; a warp's lanes differ in their odd pair, which short rows do not.
+//
+// Whole calls, us: candidate by candidate from the 16-byte positions / lone
+// slots read apart and the distances of no hit set to 0 / now, short / long:
+// the 2M-particle tank's 1.6M corners 583 / 508 / 497 / 483; a million particles
+// at 30 neighbours, h/2 cells, corners h/2 apart 350 / 431 / 347 / 372; in h
+// cells 393 / 361 / 349 / 334; 262,144 at 8 neighbours, corners 0.4 h apart,
+// radius 1.2 h 497 / 596 / 494 / 545.
+template <bool LONG>
 __global__ void __launch_bounds__(256)
 k_voxel_density(SoaPos xyz, const unsigned* __restrict__ start, Scenes sc, VoxelConst v, float* __restrict__ phi,
                 int* __restrict__ count)
@@ -277,44 +286,39 @@ k_voxel_density(SoaPos xyz, const unsigned* __restrict__ start, Scenes sc, Voxel
         const float2 t = __ffma2_rn(r2, ninv, one);
         const float2 u = make_float2(h0 ? t.x : 0.0f, h1 ? t.y : 0.0f);
         const float2 k = __fmul2_rn(__fmul2_rn(u, u), u);
-        // a candidate beyond R adds +0 (its distance is set to 0: infinity times 0 is none)
-        const float2 ex = make_float2(h0 ? dx.x : 0.0f, h1 ? dx.y : 0.0f),
-                     ey = make_float2(h0 ? dy.x : 0.0f, h1 ? dy.y : 0.0f),
-                     ez = make_float2(h0 ? dz.x : 0.0f, h1 ? dz.y : 0.0f);
+        // a candidate beyond R adds +0 (its distance is finite)
         ks = __fadd2_rn(ks, k);
-        kx = __ffma2_rn(k, ex, kx);
-        ky = __ffma2_rn(k, ey, ky);
-        kz = __ffma2_rn(k, ez, kz);
+        kx = __ffma2_rn(k, dx, kx);
+        ky = __ffma2_rn(k, dy, ky);
+        kz = __ffma2_rn(k, dz, kz);
         cnt += (int)h0 + (int)h1;
     };
     const float2* __restrict__ X2 = reinterpret_cast<const float2*>(xyz.x);
     const float2* __restrict__ Y2 = reinterpret_cast<const float2*>(xyz.y);
     const float2* __restrict__ Z2 = reinterpret_cast<const float2*>(xyz.z);
-    // a lone slot: its pair's other half at infinity
-    auto take1 = [&](unsigned j) {
-        const float a = __ldg(xyz.x + j), b = __ldg(xyz.y + j), d = __ldg(xyz.z + j);
-        const bool odd = j & 1u;
-        take2(make_float2(odd ? INFINITY : a, odd ? a : INFINITY), make_float2(b, b), make_float2(d, d));
-    };
     RowWalk walk(c.g, v.wb, start + c.c_base, x, y, z);
     unsigned s0, s1;
     while (walk.next(s0, s1)) {
-        unsigned j = s0;
-        if (j & 1u) take1(j++);
-        const unsigned e = s1 & ~1u;
-        for (; j + 4 <= e; j += 4) {  // two pairs in flight
+        unsigned j = s0 & ~1u;
+        if (LONG)
+            for (; j + 2 < s1; j += 4) {
+                const unsigned k = j >> 1;
+                float2 xa = __ldg(X2 + k), xb = __ldg(X2 + k + 1);
+                const float2 ya = __ldg(Y2 + k), za = __ldg(Z2 + k);
+                const float2 yb = __ldg(Y2 + k + 1), zb = __ldg(Z2 + k + 1);
+                if (j < s0) xa.x = HIDDEN;
+                if (j + 3 >= s1) xb.y = HIDDEN;
+                take2(xa, ya, za);
+                take2(xb, yb, zb);
+            }
+        for (; j < s1; j += 2) {
             const unsigned k = j >> 1;
-            const float2 xa = __ldg(X2 + k), ya = __ldg(Y2 + k), za = __ldg(Z2 + k);
-            const float2 xb = __ldg(X2 + k + 1), yb = __ldg(Y2 + k + 1), zb = __ldg(Z2 + k + 1);
-            take2(xa, ya, za);
-            take2(xb, yb, zb);
+            float2 X = __ldg(X2 + k);
+            const float2 Y = __ldg(Y2 + k), Z = __ldg(Z2 + k);
+            if (j < s0) X.x = HIDDEN;
+            if (j + 1 >= s1) X.y = HIDDEN;
+            take2(X, Y, Z);
         }
-        if (j < e) {
-            const unsigned k = j >> 1;
-            take2(__ldg(X2 + k), __ldg(Y2 + k), __ldg(Z2 + k));
-            j += 2;
-        }
-        if (j < s1) take1(j);
     }
     float f = v.R;
     if (cnt > 0) {
@@ -325,12 +329,19 @@ k_voxel_density(SoaPos xyz, const unsigned* __restrict__ start, Scenes sc, Voxel
     if (count) count[idx] = cnt;
 }
 
+// Candidates of a row at rest density from which LONG is taken.  Short / long,
+// us: 3.3 candidates 347 / 372, 5.2 92 / 98, 6.2 167 / 169, 6.6 99 / 102, 7.5
+// 181 / 179, 11 (the tank) 497 / 483, 17 349 / 334, 44 135 / 126.
+constexpr float LONG_ROWS = 7.0f;
+
 cudaError_t launch_voxel_density(const SoaPos& xyz, const unsigned* start, const Scenes& sc, const VoxelConst& v,
                                  float* phi, int* count, cudaStream_t s, long long* launches)
 {
     const long long n = (long long)v.dims[0] * v.dims[1] * v.dims[2];
     if (n <= 0) return cudaSuccess;
-    k_voxel_density<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(xyz, start, sc, v, phi, count);
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (v.row > LONG_ROWS) k_voxel_density<true><<<blocks, 256, 0, s>>>(xyz, start, sc, v, phi, count);
+    else k_voxel_density<false><<<blocks, 256, 0, s>>>(xyz, start, sc, v, phi, count);
     ++*launches;
     return cudaGetLastError();
 }

@@ -1268,8 +1268,8 @@ struct sph_mlp {
     unsigned* err;
     long long step;
     long long launches;
-    // tensor maps of the handle's own arrays (built by the first training call)
-    bool maps_ready;
+    // tensor maps of the handle's own arrays (built with it: its calls, from
+    // whatever thread, only read them)
     TrainMaps tmaps;
     DwMaps dmaps;
     char msg[512];
@@ -1344,9 +1344,8 @@ static int sms_of_device(sph_mlp* m, int* sms)
     return SPH_OK;
 }
 
-static int train_maps(sph_mlp* m)
+static int build_maps(sph_mlp* m)
 {
-    if (m->maps_ready) return SPH_OK;
     const ParamLayout L;
     for (int l = 0; l < 4; ++l)
         MLP_TRY(m, make_map(&m->tmaps.w[l], m->W + L.w[l], L.out[l], L.in[l], L.in[l], L.out[l]));
@@ -1357,7 +1356,6 @@ static int train_maps(sph_mlp* m)
         MLP_TRY(m, make_map(&m->dmaps.in[l], l ? m->HT[l - 1] : m->XT, L.in[l], m->max_batch, m->max_batch, dw::NT));
         MLP_TRY(m, make_map(&m->dmaps.b[l], l < 3 ? m->DT[l] : m->DYT, L.out[l], m->max_batch, m->max_batch, dw::BR));
     }
-    m->maps_ready = true;
     return SPH_OK;
 }
 
@@ -1380,8 +1378,7 @@ static int launch_rows(sph_mlp* m, const CUtensorMap& mx, const TrainArgs& a, cu
 static int mlp_forward_fused(sph_mlp* m, const __nv_bfloat16* x, int B, float* y, cudaStream_t s)
 {
     CUtensorMap mx;
-    int sms = 0, rc = train_maps(m);
-    if (rc == SPH_OK) rc = sms_of_device(m, &sms);
+    int sms = 0, rc = sms_of_device(m, &sms);
     if (rc != SPH_OK) return rc;
     // Few rows: 16 or 32 a CTA instead of 128, so that more of the chip works
     // on them: 128 to 2,432 rows take 14 us instead of 22, up to 4,864 rows
@@ -1420,8 +1417,7 @@ static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const 
                       float* grads, const AdamArgs* adam, float* loss, cudaStream_t s)
 {
     const ParamLayout L;
-    int rc = train_maps(m), sms = 0;
-    if (rc == SPH_OK) rc = sms_of_device(m, &sms);
+    int sms = 0, rc = sms_of_device(m, &sms);
     if (rc != SPH_OK) return rc;
     TrainArgs a;
     memset(&a, 0, sizeof(a));
@@ -1509,6 +1505,11 @@ int sph_mlp_create(int max_batch, void* workspace, size_t ws_bytes, sph_mlp** ou
     if (e != cudaSuccess) {
         delete m;
         return mfail(nullptr, SPH_ERR_CUDA, "cudaMemset: %s", cudaGetErrorString(e));
+    }
+    rc = build_maps(m);
+    if (rc != SPH_OK) {
+        delete m;
+        return rc;
     }
     *out = m;
     return SPH_OK;

@@ -1,5 +1,5 @@
-"""The network called from other host threads than the one that made it (needs
-a GB300)."""
+"""The network called from other host threads than the one that made it, and from
+several at once (needs a GB300)."""
 import threading
 
 import numpy as np
@@ -10,6 +10,8 @@ from oracle import mlp as omlp
 from paper_2311_15088_gb300 import sph
 
 pytestmark = pytest.mark.gpu
+
+THREADS = 4
 
 
 def _packed():
@@ -52,3 +54,35 @@ def test_first_cuda_call_of_a_thread(call):
         out += [o, m.get_params()]
     assert rc == [0, 0]
     assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3]) and bool(out[0].any())
+
+
+# rows for 16 and 32 rows a CTA and for the 128-row tiles
+@pytest.mark.parametrize("rows_per_sm", [4, 20, 40])
+def test_first_calls_of_a_handle_from_several_threads(rows_per_sm):
+    B = rows_per_sm * torch.cuda.get_device_properties(0).multi_processor_count // 128 * 128
+    packed = _packed()
+    g = torch.Generator(device="cuda").manual_seed(B)
+    x = [torch.randn((B, sph.SPH_MLP_IN), generator=g, device="cuda").to(torch.bfloat16) for _ in range(THREADS)]
+    m = sph.Mlp(B)
+    m.set_params(packed)
+    want = [m.forward(v) for v in x]
+    streams = [torch.cuda.Stream() for _ in range(THREADS)]
+    for _ in range(8):
+        m = sph.Mlp(B)
+        m.set_params(packed)
+        torch.cuda.synchronize()
+        got, start = [None] * THREADS, threading.Barrier(THREADS)
+
+        def first_call(k):
+            with torch.cuda.stream(streams[k]):
+                start.wait()
+                got[k] = m.forward(x[k])
+
+        threads = [threading.Thread(target=first_call, args=(k,)) for k in range(THREADS)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize()
+        assert m.status() == 0
+        assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -1216,7 +1216,7 @@ k_train_update(const float* __restrict__ part, int splits, int lo, float* __rest
     }
     *reinterpret_cast<float4*>(G + t) = make_float4(g[0], g[1], g[2], g[3]);
     if (grads)
-        for (int e = 0; e < 4; ++e) grads[t + e] = g[e];  // the caller's array, of any alignment
+        for (int e = 0; e < 4; ++e) grads[t + e] = g[e];  // the caller's array, aligned as floats
     if (!adam) return;
     const int l = t >= L.w[3] ? 3 : (t >= L.w[2] ? 2 : (t >= L.w[1] ? 1 : 0));
     const int e0 = t - L.w[l], nin = l == 0 ? MLP_IN : MLP_H, nout = l == 3 ? MLP_OUT : MLP_H;
@@ -1460,11 +1460,17 @@ static int train_pass(sph_mlp* m, const __nv_bfloat16* x, const float* t, const 
     k_train_dw<<<dim3(dw::TILES - first + nbias, splits), 160, dw::TOTAL, s>>>(m->dmaps, first, kb, per, m->part, m->err);
     AdamArgs none;
     memset(&none, 0, sizeof(none));
+    // the kernel writes the caller's floats itself where they are aligned as
+    // floats; elsewhere they are copied from the handle's
+    auto aligned = [](float* p) { return ((uintptr_t)p & 3) == 0; };
     k_train_update<<<(SPH_MLP_PARAMS - lo + 511) / 512, 128, 0, s>>>(
-        m->part, splits, lo, m->G, grads, adam != nullptr, adam ? *adam : none, m->P, m->Mo, m->Vo, m->W, m->WT,
-        m->loss_part, 2 * (B / NB), B, loss);
+        m->part, splits, lo, m->G, aligned(grads) ? grads : nullptr, adam != nullptr, adam ? *adam : none, m->P, m->Mo,
+        m->Vo, m->W, m->WT, m->loss_part, 2 * (B / NB), B, aligned(loss) ? loss : m->loss);
     m->launches += 2;
     MLP_TRY(m, cudaGetLastError());
+    if (!aligned(grads))
+        MLP_TRY(m, cudaMemcpyAsync(grads, m->G, sizeof(float) * SPH_MLP_PARAMS, cudaMemcpyDeviceToDevice, s));
+    if (!aligned(loss)) MLP_TRY(m, cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToDevice, s));
     return SPH_OK;
 }
 

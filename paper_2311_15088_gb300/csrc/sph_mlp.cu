@@ -181,6 +181,17 @@ struct GemmSmem {
     static constexpr uint32_t TMEM_COLS = NT < 32 ? 32 : NT;
 };
 
+// For the consumer of a ring of stages that gave up at copy `first` of `total`:
+// let the copies that may be in flight by then land, within the waits' limit.
+// The loader may have issued its last ones and be done, and the block must not
+// go away under them; a loader that gives up waits for its own.
+// (Out of line, so that the kernels' loops are compiled as without it.)
+__device__ __noinline__ void drain_ring(int stages, int first, int total, uint32_t full0, unsigned* err)
+{
+    for (int i = first; i < min(total, first + stages); ++i)
+        mbar_wait(full0 + 8u * (uint32_t)(i % stages), (uint32_t)(i / stages) & 1u, err);
+}
+
 // One CTA of 128 threads per (M tile, N tile, K split).  Warp 0 lane 0
 // streams the A and B tiles through a STAGES-deep TMA ring, warp 1 lane 0
 // issues the tcgen05.mma and frees each stage with tcgen05.commit, and all
@@ -248,7 +259,10 @@ k_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtenso
         constexpr uint32_t idesc = umma_idesc_bf16(BM, NT);
         for (int i = 0; i < nk; ++i) {
             const int s = i % STAGES;
-            if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, e.err)) break;
+            if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, e.err)) {
+                drain_ring(STAGES, i, nk, full(0), e.err);
+                break;
+            }
             tc_fence_after();
             const uint32_t a = tiles + (uint32_t)s * L::STAGE;
             const uint32_t b = a + L::A_BYTES;
@@ -587,6 +601,7 @@ k_mlp_fused(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CU
             if (!ok) {  // so that the epilogue does not wait for nothing
                 umma_commit(acc_full(0));
                 umma_commit(acc_full(1));
+                drain_ring(STAGES, g, ntl * (KB_IN + 3 * KB_H), full(0), err);
             }
         }
     } else {
@@ -841,7 +856,12 @@ k_train_rows(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ T
                 if (!ok) break;
                 umma_commit(acc_full);
             }
-            if (!ok) umma_commit(acc_full);  // so that the epilogue does not wait for nothing
+            if (!ok) {
+                umma_commit(acc_full);  // so that the epilogue does not wait for nothing
+                int total = 0;
+                for (int s = 0; s < nsteps; ++s) total += kblocks(s);
+                drain_ring(STAGES, g, total, full(0), a.err);
+            }
         }
     } else {
         // warp w reads tensor-memory lanes 32 (w % 4) ..; part w / 4 picks the
@@ -1080,13 +1100,15 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
         };
         bool ok = wait(0);
         if (ok) fetch(0, 0);
-        for (int i = 0; ok && i < n; ++i) {
+        int i = 0;
+        for (; ok && i < n; ++i) {
             fetch(i, 1);
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty(i % BIAS_STAGES)) : "memory");
             sum(v[0]);
             if (i + 1 < n && (ok = wait(i + 1))) fetch(i + 1, 0);
             sum(v[1]);
         }
+        if (!ok) drain_ring(BIAS_STAGES, i, n, full(0), err);
         const int f = m0 + lane;
         if (ok && f < L.out[l])  // the other slices hold zeros
             for (int k = 0; k < (int)gridDim.y; ++k) part[(size_t)k * SPH_MLP_PARAMS + L.b[l] + f] = k ? 0.0f : s;
@@ -1123,7 +1145,10 @@ k_train_dw(const __grid_constant__ DwMaps maps, int first_tile, int kb_total, in
         constexpr uint32_t idesc = umma_idesc_bf16(BM, NT);
         for (int i = 0; i < nk; ++i) {
             const int s = i % STAGES;
-            if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, err)) break;
+            if (!mbar_wait(full(s), (uint32_t)(i / STAGES) & 1u, err)) {
+                drain_ring(STAGES, i, nk, full(0), err);
+                break;
+            }
             tc_fence_after();
             const uint32_t a = base + s * STAGE, b = a + A_BYTES;
 #pragma unroll

@@ -184,7 +184,11 @@ int sph_batch_create(const sph_params* params, const int* n_fluid, const int* n_
  * candidates again (1 KiB of workspace per particle holds them; a
  * particle with more than 128 segments is tested again).  use_segments = 0:
  * the force pass tests the candidates itself.  Neither choice changes any
- * result bit: the pairs and their order are the same.  Errors: SPH_ERR_ARG.
+ * result bit: the pairs and their order are the same.  Launches of few
+ * particles take them with a warp each, in blocks of their own: the density
+ * pass up to 108 particles per multiprocessor of the device, the force pass
+ * (with segments, without neighbour lists) up to 80; `block` acts on the
+ * passes above those.  Errors: SPH_ERR_ARG.
  */
 int sph_set_tuning(sph_handle* h, int block, int use_segments);
 
@@ -192,7 +196,8 @@ int sph_set_tuning(sph_handle* h, int block, int use_segments);
  * Particles per thread of the two neighbour passes' separate launches (the
  * trade-off of section "Experimental Results": fewer threads, each taking
  * several particles): ppt = 1 (the default), 2 or 4; thread t of a grid of
- * T threads takes particles t, t + T, ...  No result bit changes.  The fused
+ * T threads takes particles t, t + T, ...  No result bit changes.  It acts on
+ * the passes that take a thread per particle (see sph_set_tuning); the fused
  * pipeline (sph_set_pipeline) takes its own tiles.  Errors: SPH_ERR_ARG.
  */
 int sph_set_particles_per_thread(sph_handle* h, int ppt);
@@ -262,9 +267,9 @@ int sph_get_state(sph_handle* h, float* fluid_pos4, float* fluid_vel4,
  * v_b += sph_factor dt F_b, edge avoidance, speed limit, x_b += v_b dt);
  * Euler-Cromer integration of the fluid with damped wall reflection.
  * With boids (and without the fused pipeline of sph_set_pipeline), the
- * boids' binning, F_b and rules run on a stream the handle owns, forked from
- * `stream` at the start of each step and joined back into it before the
- * step ends: to the caller the work is ordered on `stream` as if it ran
+ * boids' binning runs on a stream the handle owns, forked from `stream` at the
+ * start of each step and joined back into it before the force pass, whose
+ * launch also computes F_b and applies the rules: to the caller the work is ordered on `stream` as if it ran
  * there alone (a capture of `stream` takes the side branch with it), and the
  * results are bit for bit those of the serial order.
  * Errors: SPH_ERR_ARG (nsteps < 0), SPH_ERR_STATE (no state loaded),

@@ -11,7 +11,7 @@
 //
 // Every boid reads the start-of-step snapshot (sorted copies), so the result
 // does not depend on the order boids are processed in.  Lanes stride over
-// the candidates of the boid cells within r_vis (RowWalk) and the warp
+// the candidates of the boid cells within r_vis (WarpRows) and the warp
 // sums with a fixed butterfly, so the float32 result is deterministic.
 #include "sph_boids.cuh"
 

@@ -192,6 +192,8 @@ __device__ __noinline__ void drain_ring(int stages, int first, int total, uint32
         mbar_wait(full0 + 8u * (uint32_t)(i % stages), (uint32_t)(i / stages) & 1u, err);
 }
 
+// A product by itself, C = A B^T: only sph_debug_gemm launches it (the network
+// runs in k_mlp_fused and k_train_*).
 // One CTA of 128 threads per (M tile, N tile, K split).  Warp 0 lane 0
 // streams the A and B tiles through a STAGES-deep TMA ring, warp 1 lane 0
 // issues the tcgen05.mma and frees each stage with tcgen05.commit, and all

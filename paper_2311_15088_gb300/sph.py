@@ -695,7 +695,8 @@ class Scene:
         self.tuning = (int(block), int(use_segments))
 
     def set_particles_per_thread(self, ppt: int):
-        """Particles per thread of the separate neighbour-pass launches."""
+        """Particles per thread of the separate neighbour-pass launches (those
+        too large for a warp per particle)."""
         sph_set_particles_per_thread(self.handle, ppt)
         self.ppt = int(ppt)
 

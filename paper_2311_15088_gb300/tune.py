@@ -7,6 +7,9 @@ its pairs from the density pass's hit segments or tests the candidates
 again; for the fused
 persistent pipeline (both passes in one cooperative launch over work items),
 the sorted slots per work item (a run of cells) and the threads per CTA.
+Scenes of few particles take a warp per particle whatever the block and the
+particles per thread (sph_set_tuning): their shapes with segments are one
+launch shape, and the choice among them is that of the timings' noise.
 For a scene (or batch) the tuner snapshots the state, times a few steps of
 each candidate shape with CUDA events, restores the state, applies the
 fastest shape and caches the choice in a JSON file keyed by the workload's

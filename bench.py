@@ -97,9 +97,9 @@ BYTES_PER_CELL_SCAN = 12
 # fluid particles, F_b and the boid rules in one launch).
 KERNEL_TRAFFIC = {
     "k_forces": {"bytes": 742.6e6, "read": 653.3e6, "write": 89.3e6,
-                 "source_sha256": "2248f66d7e3f6521b8468678b22cfdd775610939ff93ca9e4ab76ac92c74a990"},
-    "k_density": {"bytes": 865.5e6, "read": 290.3e6, "write": 575.3e6,
-                  "source_sha256": "2248f66d7e3f6521b8468678b22cfdd775610939ff93ca9e4ab76ac92c74a990"},
+                 "source_sha256": "b8cf74fa338c321f5af4f6d69fc3e3444a6646bafbc656ef705b3538d6332150"},
+    "k_density": {"bytes": 868.0e6, "read": 291.6e6, "write": 576.4e6,
+                  "source_sha256": "b8cf74fa338c321f5af4f6d69fc3e3444a6646bafbc656ef705b3538d6332150"},
 }
 
 

@@ -241,6 +241,8 @@ k_scan_tiles(unsigned* __restrict__ in, int n, const unsigned* __restrict__ part
 // Two launches up to this many tiles (33.5M cells; the large tank's grid has
 // 1,430): a block adds up to 32 totals per thread.  As three launches and a
 // fourth for the grand total the scan was a quarter of a small step's chain.
+// A step of 2,000 particles in grids of 1,500, 6,000 and 8,191 tiles takes 32,
+// 89 and 114 us (80, 134 and 165 with the four), of 9,000, with three, 122 (169).
 constexpr int SCAN_SUM_MAX = 8192;
 
 cudaError_t launch_scan(unsigned* counts, int n, unsigned* part, unsigned* start, bool zero, cudaStream_t s,

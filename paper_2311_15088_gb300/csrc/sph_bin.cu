@@ -405,7 +405,8 @@ cudaError_t launch_cellsort_slots(const unsigned* start, const unsigned* key, in
 __global__ void __launch_bounds__(256)
 k_slot_keys(const unsigned* __restrict__ start, int ncells, unsigned* __restrict__ slot_key)
 {
-    int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // (a grid of more than 2^27 cells has more threads than 32 bits count)
+    const int c = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     int lane = threadIdx.x & 31;
     if (c >= ncells) return;
     for (unsigned s = start[c] + lane; s < start[c + 1]; s += 32) slot_key[s] = (unsigned)c;

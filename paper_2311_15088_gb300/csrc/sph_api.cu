@@ -1376,6 +1376,8 @@ int sph_get_fields(sph_handle* h, int field, void* out, int on_host, void* strea
         break;
     case SPH_FIELD_BOID_CELL_START:
         bytes = ((size_t)h->nbcells + 1) * 4;
+        // without boids nothing is binned: every cell starts at 0
+        if (!nb) CUDA_TRY(h, cudaMemsetAsync(h->bstart, 0, bytes, s));
         CUDA_TRY(h, cudaMemcpyAsync(out, h->bstart, bytes, on_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s));
         if (on_host) CUDA_TRY(h, cudaStreamSynchronize(s));
         return SPH_OK;
